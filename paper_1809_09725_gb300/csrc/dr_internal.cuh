@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <string>
@@ -146,6 +147,29 @@ enum RedSlot {
     kSlotDot = 7,
 };
 
+// A table of rows of ms coefficients, one per (slice, distinct angle, bin):
+// row (z, a, b) starts at (z / spb) blk + (a ns + b) C + (z % spb) ms floats.
+// spb = 1 and C = ms is the slice-major layout of the thread-per-ray kernels;
+// the channel layout packs spb slices side by side into blocks of C channels.
+struct RowMap {
+    int spb, C, ms;
+    size_t blk;
+};
+
+// Channel-lane folded projectors (chan.cuh) of a plan: geometry of the launch,
+// work lists, scratch.  V = 0: not available.
+struct ChanPlan {
+    int V = 0, C = 0, ms = 0, spb = 0, ncb = 0;  // channels per lane / block, row length, slices per block, blocks
+    int nw = 0, n = 0, g = 0, nblocks = 0, nbx = 0;  // warps, angles x runs of bins per CTA; angle blocks, bin blocks
+    int nsplit = 1, cb_pass = 1;                 // line chunks; channel blocks packed at a time
+    int fwd = 0, fwd_st = 0;                     // chosen by the autotuner (compute-typed / bf16-stored calls)
+    int *d_blocks = nullptr;
+    RowMap rows{};
+    size_t gt_bytes = 0, uc_bytes = 0;           // table of rows / packed volume
+    void *d_gt = nullptr, *d_uc = nullptr;
+    size_t gt_held = 0, uc_held = 0;
+};
+
 struct Workspace {
     size_t bytes = 0;
     dr_algo algo = DR_ADMM_CG;
@@ -231,6 +255,7 @@ struct dr_plan {
     void *d_ru_split = nullptr;       // partial sums of a split march (allocated on first use)
     size_t ru_split_bytes = 0;
     int fold2_lines = 1, fold2_lines_st = 1;  // strip lines (compute-typed / bf16 kernels)
+    dr::ChanPlan chan;
     void *d_gt = nullptr;             // folded data [nz][U][ns][MS] float (allocated on first use)
     size_t gt_bytes = 0;
     int var_fwd = -1, var_adj = -1;   // -1 automatic, 0 direct, 1 fold, 2 fold in two kernels (forward)
@@ -265,6 +290,18 @@ inline size_t nvox(const dr_plan *P) { return (size_t)P->nx * P->ny * P->nz; }
 inline size_t nu_elems(const dr_plan *P) { return nvox(P) * P->m; }
 inline size_t ng_elems(const dr_plan *P) { return (size_t)P->nz * P->K * P->ns; }
 inline size_t nf_elems(const dr_plan *P) { return nvox(P) * P->nt * 4; }
+
+// What a serving job's memory estimate counts for the folded projectors: the
+// folded data (at most one distinct angle per projection), and the partial sums
+// of a split march.  Their scratch stays within it (the estimate knows K, not
+// the number of distinct angles).
+inline size_t fold_budget(int nz, int K, int ns, int M) {
+    const int MS = M <= 4 ? 4 : ((M % 8 == 0) ? M + 4 : M);
+    return sizeof(float) * (size_t)nz * K * ns * MS;
+}
+inline size_t split_budget(int nz, int K, int ns, int m) {
+    return std::min<size_t>(size_t(256) << 20, 4 * sizeof(float) * (size_t)nz * K * ns * ((m + 3) / 4 * 4));
+}
 
 inline int red_grid(size_t n) {
     size_t b = (n + kRedThreads - 1) / kRedThreads;

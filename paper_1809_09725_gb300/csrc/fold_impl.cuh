@@ -22,7 +22,7 @@
 #pragma once
 #include <type_traits>
 
-#include "dr_device.cuh"
+#include "chan.cuh"
 
 namespace dr {
 
@@ -515,7 +515,7 @@ template <typename S, typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
     fold_dist_kernel(const T *__restrict__ ru, S *__restrict__ out, const S *__restrict__ gm,
                      const int *__restrict__ start, const int *__restrict__ member, const T *__restrict__ phip,
-                     int nz, int K, int ns, int U, int ms_ru, int m, int MP, int mode, T sigma, int nsplit,
+                     int nz, int K, int ns, int U, RowMap rows, int m, int MP, int mode, T sigma, int nsplit,
                      size_t split_stride) {
     // rows and table rows are multiples of 4 floats from 16-byte aligned bases
     constexpr bool V4 = sizeof(T) == 4;
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kRedThreads)
         const int b = (int)(i % ns);
         const size_t za = i / ns;
         const int a = (int)(za % U), z = (int)(za / U);
-        const T *r = ru + i * ms_ru;
+        const T *r = ru + row_at(rows, z, (size_t)a * ns + b);
         T rv[M];
         if constexpr (V4 && M % 4 == 0) {
 #pragma unroll
@@ -909,16 +909,9 @@ dr_status fold_fwd_launch_t(dr_plan *P, const void *u, void *out, const void *gm
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "fold_fwd_kernel launch");
 }
 
-// Two-kernel folded forward: static transforms of coefficient groups of MC
-// (4 or 8) into the folded-data scratch, then the distribution.
-// Static transforms of the two-kernel forward (step 1), into the folded-data
-// scratch (one march) or the split scratch (line chunks); `rs` says where.
-struct StaticOut {
-    void *ru;
-    int ms_ru, nsplit;
-    size_t split_stride;
-};
-
+// Static transforms of the two-kernel forward (step 1) in coefficient groups
+// of MC (4 or 8): into the folded-data scratch (one march) or the split
+// scratch (line chunks); `rs` says where.
 template <typename S, typename T, int M, int GI>
 dr_status fold_static_launch(dr_plan *P, const void *u, cudaStream_t st, StaticOut &rs) {
     constexpr int MC = fold_static_mc(GI), THREADS = fold_static_threads(GI), RPT = fold_static_rpt_gi(GI),
@@ -1014,7 +1007,7 @@ dr_status fold_static_launch(dr_plan *P, const void *u, cudaStream_t st, StaticO
                                            split_stride, tm_rows, tm_cols, P->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_fwd_kernel (static) launch");
-    rs = StaticOut{ru, ms_ru, nsplit, split_stride};
+    rs = StaticOut{ru, slice_rows((size_t)P->fold_U * P->ns, ms_ru), nsplit, split_stride};
     return DR_OK;
 }
 
@@ -1044,17 +1037,19 @@ dr_status fold_static_dispatch(dr_plan *P, const void *u, cudaStream_t st, Stati
     return fail(DR_EINVAL, "two-kernel folded forward: unsupported coefficient group");
 }
 
+// The forward in two steps: static transforms (chan: of the channel kernel),
+// then the distribution.
 template <typename S, typename T, int M>
 dr_status fold_fwd2_launch_t(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                             cudaStream_t st) {
+                             cudaStream_t st, bool chan) {
     StaticOut rs{};
     {
-        dr_status s = fold_static_dispatch<S, T, M>(P, u, st, rs);
+        dr_status s = chan ? chan_static(P, u, sizeof(S) == 2, st, rs) : fold_static_dispatch<S, T, M>(P, u, st, rs);
         if (s != DR_OK) return s;
     }
     fold_dist_kernel<S, T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const T *)rs.ru, (S *)out, (const S *)gm, P->d_fold_start, P->d_fold_member, (const T *)P->d_PhiP, P->nz,
-        P->K, P->ns, P->fold_U, rs.ms_ru, P->m, P->MP, mode, (T)sigma, rs.nsplit, rs.split_stride);
+        P->K, P->ns, P->fold_U, rs.rows, P->m, P->MP, mode, (T)sigma, rs.nsplit, rs.split_stride);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "fold_dist_kernel launch");
 }
@@ -1214,8 +1209,8 @@ dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t 
         if (s != DR_OK) return s;
     }
     fold_gram_kernel<T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
-        (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.ms_ru, P->m, rs.nsplit,
-        rs.split_stride);
+        (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows.ms, P->m,
+        rs.nsplit, rs.split_stride);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_gram_kernel launch");
     return fold_backproject<S, T, M>(P, y, 1.0, 0.0, true, st);
@@ -1226,7 +1221,7 @@ struct FoldOps {
     static dr_status fwd(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                          cudaStream_t st);
     static dr_status fwd2(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                          cudaStream_t st);
+                          cudaStream_t st, bool chan = false);
     static dr_status adj(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
                          cudaStream_t st);
     // y = R*R x on compute-typed buffers (static transforms, Gram mix, back-projection)
@@ -1254,8 +1249,8 @@ dr_status FoldOps<S, T>::fwd(dr_plan *P, const void *u, void *out, const void *g
 
 template <typename S, typename T>
 dr_status FoldOps<S, T>::fwd2(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                              cudaStream_t st) {
-    DR_FOLD_DISPATCH(fold_fwd2_launch_t, S, T, P, u, out, gm, mode, sigma, st)
+                              cudaStream_t st, bool chan) {
+    DR_FOLD_DISPATCH(fold_fwd2_launch_t, S, T, P, u, out, gm, mode, sigma, st, chan)
 }
 
 template <typename S, typename T>

@@ -10,6 +10,7 @@
 #include <mutex>
 #include <string>
 
+#include "chan.cuh"
 #include "dr_device.cuh"
 #include "dr_internal.cuh"
 
@@ -503,6 +504,10 @@ static dr_status build_tables(dr_plan *P) {
         // default: groups of 4 coefficients, 256 threads (the autotuner times all)
         P->fold2_gi = P->fold2_gi_st = 0;
         P->fold2_lines = P->fold2_lines_st = std::max(1, std::min(4, P->fold2_R[0]));
+        {
+            dr_status s = chan_setup(P, ufw);
+            if (s != DR_OK) return s;
+        }
         // cost model until measured: fold when the unique angles carry the work
         const double direct = (double)K * (P->m + 16), fold = (double)U * (3.0 * P->m + 12) + 0.05 * K * P->m;
         P->sel_fwd = (P->fold_fwd_ok && fold < 0.8 * direct) ? 1 : 0;
@@ -624,6 +629,7 @@ dr_status dr_plan_destroy(dr_plan *P) {
                     P->d_fbp_u, P->d_ru_split, P->d_fold_gram};
     for (void *p : ptrs)
         if (p) cudaFree(p);
+    chan_free(P);
     for (auto &row : P->d_fold2_blocks)
         for (int *p : row)
             if (p) cudaFree(p);
@@ -641,7 +647,8 @@ dr_status dr_plan_set_stream(dr_plan *P, void *s) {
 }
 
 size_t dr_plan_device_bytes(const dr_plan *P) {
-    return P ? P->table_bytes + P->ws.bytes + (P->d_gt ? P->gt_bytes : 0) + P->fbp_bytes + P->ru_split_bytes : 0;
+    return P ? P->table_bytes + P->ws.bytes + (P->d_gt ? P->gt_bytes : 0) + P->fbp_bytes + P->ru_split_bytes +
+                   P->chan.gt_held + P->chan.uc_held : 0;
 }
 
 }  // extern "C"

@@ -50,6 +50,15 @@ dr_status launch_fwd_variant(dr_plan *P, int variant, bool calc, const void *u, 
         if (P->prec == DR_BF16_F32ACC && !calc) return FoldOps<bf16, float>::fwd(P, u, out, gm, mode, sigma, st);
         return FoldOps<float, float>::fwd(P, u, out, gm, mode, sigma, st);
     }
+    if (variant == kVarChan) {
+        if (chan_fwd_ready(P, st)) {
+            if (P->prec == DR_BF16_F32ACC && !calc)
+                return FoldOps<bf16, float>::fwd2(P, u, out, gm, mode, sigma, st, true);
+            return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st, true);
+        }
+        // no scratch to be had (memory, a capture, a slab's budget)
+        variant = calc || P->prec != DR_BF16_F32ACC ? P->sel_fwd : P->sel_fwd_st;
+    }
     if (variant == 2 && P->fold_U > 0 && P->fold2_ok) {
         if (P->prec == DR_BF16_F32ACC && !calc) return FoldOps<bf16, float>::fwd2(P, u, out, gm, mode, sigma, st);
         return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st);
@@ -83,10 +92,17 @@ dr_status launch_adj_variant(dr_plan *P, int variant, bool calc, const void *g, 
     return fail(DR_EINVAL, "bad precision");
 }
 
+// ADMM's forwards: its CG steps amplify the rounding of every sum, so the solver
+// keeps to the thread-per-ray kernels, whose sums it has always used, and its
+// iterates and objective stay what they are, bit for bit, whichever kernel is
+// the fastest one for a single call.
 static int fwd_choice(const dr_plan *P) { return P->var_fwd >= 0 ? P->var_fwd : P->sel_fwd; }
 // storage-typed calls on BF16 plans run the bf16-strip kernels, timed separately
 static int fwd_choice_st(const dr_plan *P) {
-    return P->var_fwd >= 0 ? P->var_fwd : (P->prec == DR_BF16_F32ACC ? P->sel_fwd_st : P->sel_fwd);
+    if (P->var_fwd >= 0) return P->var_fwd;
+    const bool st = P->prec == DR_BF16_F32ACC;
+    if (st ? P->chan.fwd_st : P->chan.fwd) return kVarChan;
+    return st ? P->sel_fwd_st : P->sel_fwd;
 }
 static int adj_choice(const dr_plan *P) { return P->var_adj >= 0 ? P->var_adj : P->sel_adj; }
 
@@ -105,6 +121,13 @@ dr_status launch_adj(dr_plan *P, const void *g, void *u, double alpha, double be
 dr_status launch_fwd_calc(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                           cudaStream_t st) {
     return launch_fwd_variant(P, fwd_choice(P), true, u, out, gm, mode, sigma, st);
+}
+
+// Chambolle-Pock's forwards (no inner products: rounding is not amplified).
+dr_status launch_fwd_cp(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
+                        cudaStream_t st) {
+    const int v = P->var_fwd < 0 && P->chan.fwd ? kVarChan : fwd_choice(P);
+    return launch_fwd_variant(P, v, true, u, out, gm, mode, sigma, st);
 }
 
 dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, double beta, cudaStream_t st) {
@@ -132,16 +155,16 @@ dr_status launch_normal_calc(dr_plan *P, const void *x, void *y, void *gscratch,
 // angles and times), so every plan of the same problem runs the same
 // kernels and produces bit-identical results.
 struct TuneKey {
-    int nx, ny, nz, ns, K, m, nt, basis, prec;
+    int nx, ny, nz, ns, K, m, nt, basis, prec, slab;
     uint64_t hash;
     bool operator<(const TuneKey &o) const {
-        return std::tie(nx, ny, nz, ns, K, m, nt, basis, prec, hash) <
-               std::tie(o.nx, o.ny, o.nz, o.ns, o.K, o.m, o.nt, o.basis, o.prec, o.hash);
+        return std::tie(nx, ny, nz, ns, K, m, nt, basis, prec, slab, hash) <
+               std::tie(o.nx, o.ny, o.nz, o.ns, o.K, o.m, o.nt, o.basis, o.prec, o.slab, o.hash);
     }
 };
 struct TuneVal {
     int fwd, adj, lines, async, lines_st, async_st, f2_gi, f2_lines, f2_lines_st, fwd_st, f2_split, f2_async,
-        f2_async_st, adj_pp, f2_bv, f2_gi_st;
+        f2_async_st, adj_pp, f2_bv, f2_gi_st, chan_fwd, chan_fwd_st;
     double ms[5];
 };
 static std::mutex g_tune_mutex;
@@ -155,7 +178,7 @@ static TuneKey tune_key(const dr_plan *P) {
     };
     mix(P->theta);
     mix(P->t);
-    return TuneKey{P->nx, P->ny, P->nz, P->ns, P->K, P->m, P->nt, (int)P->basis, (int)P->prec, h};
+    return TuneKey{P->nx, P->ny, P->nz, P->ns, P->K, P->m, P->nt, (int)P->basis, (int)P->prec, (int)P->split_off, h};
 }
 
 dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
@@ -184,6 +207,8 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
             P->fold2_async_st = it->second.f2_async_st;
             P->fold_adj_pp = it->second.adj_pp;
             P->fold2_bv = it->second.f2_bv;
+            P->chan.fwd = it->second.chan_fwd;
+            P->chan.fwd_st = it->second.chan_fwd_st;
             for (int i = 0; i < 5; ++i) P->tune_ms[i] = it->second.ms[i];
             P->tuned = true;
             return DR_OK;
@@ -204,7 +229,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
     DR_CUDA_TRY(cudaMemsetAsync(u_scratch, 0, nu_elems(P) * cs, st));
     DR_CUDA_TRY(cudaMemsetAsync(g_scratch, 0, ng_elems(P) * cs, st));
     double ms[5] = {1e30, 1e30, 1e30, 1e30, 1e30};
-    double ms_st1 = 1e30, ms_st2 = 1e30;  // bf16-strip kernels of BF16 plans: fold, fold in two kernels
+    double ms_st0 = 1e30, ms_st1 = 1e30, ms_st2 = 1e30;  // bf16-strip kernels of BF16 plans: direct, fold, fold in two
     // launches per trial: one warm-up, then the timed ones (reps - 1; the
     // screening trials and the direct variant, timed only for comparison, take one)
     // a serving job canceled while its plan is being tuned stops between trials
@@ -552,7 +577,6 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
     }
     if (P->prec == DR_BF16_F32ACC) {
         // storage-typed calls of BF16 plans run the bf16-strip kernels: their own choice
-        double ms_st0 = 1e30;
         dr_status s0 = time_fwd(0, ms_st0, false, 2);
         if (s0 != DR_OK) return s0;
         int best = 0;
@@ -595,6 +619,20 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         }
         P->fold_adj_pp = best_pp;
     }
+    // the channel kernel against the fastest of the others
+    P->chan.fwd = P->chan.fwd_st = 0;
+    if (chan_fwd_ready(P, st)) {
+        double t = 1e30;
+        dr_status s = time_fwd(kVarChan, t);
+        if (s != DR_OK) return s;
+        P->chan.fwd = t < std::min(ms[0], std::min(ms[1], ms[4]));
+        if (P->prec == DR_BF16_F32ACC) {  // (packs the stored values as floats)
+            t = 1e30;
+            s = time_fwd(kVarChan, t, false);
+            if (s != DR_OK) return s;
+            P->chan.fwd_st = t < std::min(ms_st0, std::min(ms_st1, ms_st2));
+        }
+    }
     for (int i = 0; i < 5; ++i) P->tune_ms[i] = ms[i] < 1e29 ? ms[i] : -1.0;
     {
         int best = 0;
@@ -610,7 +648,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
                                                  P->fold_lines_st, P->fold_async_st, P->fold2_gi, P->fold2_lines,
                                                  P->fold2_lines_st, P->sel_fwd_st, P->fold2_split,
                                                  P->fold2_async, P->fold2_async_st, P->fold_adj_pp, P->fold2_bv,
-                                                 P->fold2_gi_st, {0, 0, 0, 0, 0}});
+                                                 P->fold2_gi_st, P->chan.fwd, P->chan.fwd_st, {0, 0, 0, 0, 0}});
     if (ins.second) {
         for (int i = 0; i < 5; ++i) ins.first->second.ms[i] = P->tune_ms[i];
     } else {  // another thread tuned the same problem first: follow its choice
@@ -630,6 +668,8 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->fold2_async_st = ins.first->second.f2_async_st;
         P->fold_adj_pp = ins.first->second.adj_pp;
         P->fold2_bv = ins.first->second.f2_bv;
+        P->chan.fwd = ins.first->second.chan_fwd;
+        P->chan.fwd_st = ins.first->second.chan_fwd_st;
     }
     return DR_OK;
 }
@@ -762,7 +802,7 @@ dr_status dr_plan_info(const dr_plan *P, dr_plan_info_t *info) {
     if (!P || !info) return fail(DR_EINVAL, "dr_plan_info: NULL argument");
     info->unique_angles = P->fold_U;
     info->max_group = P->fold_maxgrp;
-    info->fwd_variant = P->var_fwd >= 0 ? P->var_fwd : P->sel_fwd;
+    info->fwd_variant = P->var_fwd >= 0 ? P->var_fwd : (P->chan.fwd ? 2 : P->sel_fwd);
     info->adj_variant = P->var_adj >= 0 ? P->var_adj : P->sel_adj;
     info->tuned = P->tuned ? 1 : 0;
     info->device_bytes = P->table_bytes + P->ws.bytes + (P->d_gt ? P->gt_bytes : 0) + P->fbp_bytes +
@@ -778,7 +818,7 @@ dr_status dr_plan_info(const dr_plan *P, dr_plan_info_t *info) {
     info->fold_adj_angles = P->fold_U > 0 ? P->fold_adj_pp : 0;
     info->fold2_angles =
         P->fold2_ok ? P->fold2_P[P->fold2_gi][P->d_fold2_blocks[P->fold2_gi][P->fold2_bv] ? P->fold2_bv : 0] : 0;
-    info->fwd_variant_storage = P->var_fwd >= 0 ? P->var_fwd : P->sel_fwd_st;
+    info->fwd_variant_storage = P->var_fwd >= 0 ? P->var_fwd : (P->chan.fwd_st ? 2 : P->sel_fwd_st);
     return DR_OK;
 }
 

@@ -118,10 +118,8 @@ static size_t job_bytes(const dr_job_desc &d) {
     const size_t nf = V * d.nt * 4;
     size_t b = plan_table_bytes(d);
     if (d.prec != DR_F64) {
-        const int MS = M <= 4 ? 4 : ((M % 8 == 0) ? M + 4 : M);
-        b += sizeof(float) * ng * MS;  // folded data (at most one distinct angle per projection)
-        // partial sums of a split two-kernel forward (the autotuner keeps them under a cap)
-        b += std::min<size_t>(kSplitScratchMax, 4 * sizeof(float) * ng * ((d.m + 3) / 4 * 4));
+        b += fold_budget(d.nz, d.K, d.ns, M);     // folded data and the folded projectors' other scratch
+        b += split_budget(d.nz, d.K, d.ns, d.m);  // partial sums of a split folded forward
     }
     const dr_algo algo = d.params.algo;
     const size_t fs = (d.prec & DR_FIELDS_BF16) ? 2 : cs;  // dual fields
