@@ -135,6 +135,21 @@ __device__ __forceinline__ void store_row(T *p, int m, const T (&v)[M]) {
         if (j < m) p[j] = v[j];
 }
 
+// Packed pairs of floats: one instruction, each half rounded by itself.
+__device__ __forceinline__ unsigned long long pack_f2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack_f2(unsigned long long v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma_f2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // Reductions.  Each block reduces NV doubles, writes them to its partial
 // slot, and the last block to finish sums all partials in a fixed order, so

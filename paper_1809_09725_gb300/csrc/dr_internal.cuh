@@ -62,6 +62,13 @@ struct AdjProj {
     double c, s, C0, inv_c;
 };
 
+// One distinct angle of the folded back-projection, with the float constants of
+// its weights.
+struct FoldAng {
+    double c, s, C0;                  // as AdjProj
+    float cf, sf, c16, e0, inv_c2, pad;  // cos, sin, 16 cos, 1/cm - 1/(2 cm^2), 1/cm^2 (cm = max(|cos|, |sin|))
+};
+
 // Adjoint tile shape: 8*VPT x 16 voxels, 128 threads, VPT voxels per thread.
 constexpr int kAdjThreads = 128;
 constexpr int kAdjTY = 16;
@@ -222,9 +229,10 @@ struct dr_plan {
     std::vector<double> h_phif, h_dphif;  // host copies of PhiF and dPhiF ([nt][MT])
     // half-turn fold (Sec. 4): projections grouped by theta mod pi
     int fold_U = 0;                   // unique angles (0: the fold is unavailable for this plan)
+    int fold_U1 = 0;                  // the first fold_U1 of them have cos >= 0 (angles ascend in [0, pi))
     int fold_maxgrp = 0;              // largest group
     dr::FwdProj *d_fold_fwd = nullptr;  // [U] Joseph constants of the unique angles
-    dr::AdjProj *d_fold_adj = nullptr;  // [U]
+    dr::FoldAng *d_fold_ang = nullptr;  // [U]
     int *d_fold_start = nullptr;      // [U+1] member ranges
     int *d_fold_member = nullptr;     // [K] 2*k + (1 if theta_k = theta0 + odd multiple of pi)
     int *d_fold_blocks = nullptr;     // [n_fold_blocks][fold_P] unique angles grouped by stepping axis

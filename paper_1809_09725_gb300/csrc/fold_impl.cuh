@@ -29,6 +29,7 @@ namespace dr {
 constexpr int kFoldThreads = 256;
 constexpr int kFoldAdjP = 8;       // unique angles per adjoint pipeline stage (default; at most 32)
 constexpr int kFoldAdjStages = 2;
+constexpr int kFoldAdjWin = 26 * 1024;  // bytes of windows per stage, at most (four CTAs per SM)
 
 // Padded coefficient stride in shared memory and in the folded data:
 // multiples of 4 floats (16-byte vectors, TMA rows) whose pattern of
@@ -662,92 +663,143 @@ __global__ void __launch_bounds__(kRedThreads)
 // ===========================================================================
 // Adjoint, step 2: voxel-driven exact transpose of the folded sinograms
 // ===========================================================================
+// A thread holds a patch of 2 x 2 voxels for MC coefficients (all M up to 16;
+// half of them, and a second thread for the rest, above) of ZS slices.  The
+// patch projects |cos| + |sin| <= sqrt 2 bins wide, so its eight taps lie in
+// four consecutive bins b .. b + 3 counted from the voxel that projects lowest:
+// that voxel takes bins 0 and 1, the two beside it two of bins 0 to 2, the one
+// across two of bins 1 to 3.  Four bin reads serve four voxels (pairs of voxels
+// took three for two), and the 11 weights, each with its exact zero where a
+// voxel has three candidates, multiply two coefficients per instruction
+// (fma.rn.f32x2, each half rounded by itself).  An added term 0 x value leaves
+// a sum of finite data as it is, so each voxel's sum is the two-tap sum, bin by
+// bin and angle by angle (ADMM amplifies any other rounding).  Angles whose sine
+// or cosine exceeds 0.99999, where the rounding of two positions could put
+// neighbouring taps two bins apart, read each voxel's two bins by themselves (a
+// CTA-uniform test per angle).
+// A quarter warp's lanes are 4 x 2 patches: their lowest bins span at most
+// 6 |cos| + 2 |sin| < 8 bins, and rows of an odd number of 16-byte slots then
+// never collide (lanes on the same bin share one broadcast).
+//
+// Positions are floats relative to the middle of a subtile of SX x 16 voxels
+// (|position| <= 18 bins: the weights are exact to about 1e-6); a tile is one
+// or two of them.
+//
+// Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.293 ms;
+// 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.60 ms.  Shared memory, 90 % busy with
+// pairs, is at 65 %; what bounds it now is issue (56 % of the slots) together
+// with the skew of a CTA's warps at the stage barrier (24 % of the stalls; three
+// stages on mbarriers without it measured 0.300 and 6.62 ms).
 struct alignas(16) FoldPrm {
-    float c, s, c8, qb;   // cos, sin, 8 cos, window-relative origin position - 1/2
-    float e0, inv_c2;     // 1/c - 1/(2c^2), 1/c^2
-    int idx_base;         // integer origin position minus the float magic
-    float c16;            // 16 cos
+    float c, s, c16, e0;  // cos, sin, 16 cos, 1/cm - 1/(2 cm^2)  (cm = max(|c|, |s|))
+    float inv_c2, pad_[3];  // 1/cm^2
+    struct {
+        float qb;  // fraction of a subtile's middle, less 1/2
+        int idx;   // its bin in the window, less the float magic
+    } sub[2];
 };
 
-// Tile of TX x kAdjTY voxels per CTA of 128 threads, VPT voxels per thread.
-// PAIRED (VPT even): a thread holds voxel pairs (x, y), (x, y+1) in VPT/2
-// columns x0 + tx + 16 v (threads 16 x 8, rows y0 + 2 ty + {0, 1}).  The two
-// voxels of a pair project sin(theta) apart, so their taps lie in three
-// consecutive bins: one read of three bins serves both (3 instead of 4 bin
-// reads per voxel and angle).  Otherwise threads 8 x 16, columns x0 + tx + 8 v.
 template <int M>
 struct FoldAdjShape {
-    static constexpr int VPT = (M <= 8) ? 4 : ((M <= 16) ? 2 : 1);
-    static constexpr int TX = 8 * VPT;
-    static constexpr bool PAIRED = (VPT % 2) == 0;
+    static constexpr int NG = M <= 16 ? 1 : 2;  // threads sharing a patch's coefficients
+    static constexpr int MC = M / NG;
+    static constexpr int TX = NG == 1 ? 32 : 16;  // tile: TX x 16 voxels per CTA of 128 threads
+    static constexpr int SX = M <= 8 ? 32 : (M <= 16 ? 16 : 8);  // subtile
+    // a row's position from the row above it (else from the subtile's middle)
+    static constexpr bool STEP = M <= 16;
+    // bins of a window: the tile's extent at any angle (35 or 22), the patch's
+    // fourth bin and a margin for the rounding of the first
+    static constexpr int WB = NG == 1 ? 41 : 28;
+    // A window is one run of WB bins x MS floats of a sinogram row, copied in
+    // boxes of at most 256 floats and whole 128-byte lines, one box row each (a
+    // box of WB rows of MS floats fetched 2.7 times the bytes from L2).
+    static constexpr int NBOX = (WB * fold_ms(M) + 255) / 256;
+    static constexpr int BOX = ((WB * fold_ms(M) + NBOX - 1) / NBOX + 31) / 32 * 32;
+    static constexpr int WIN = NBOX * BOX;  // floats
+    // slices a thread may take (the weights, about as many instructions as 8
+    // coefficients' sums, serve all of them)
+    static constexpr int ZS = M <= 4 ? 4 : (M <= 8 ? 2 : 1);
 };
 
-// Seven 128-thread CTAs per SM (<= 72 registers): with the default seven
-// angles per pipeline stage, shared memory admits seven too (M <= 16).
-__host__ __device__ constexpr int fold_adj_min_blocks(int M) { return M <= 16 ? 7 : 6; }
+// Resident CTAs asked for: 4 ZS MC sums, 11 weight pairs and 4 bins per thread.
+__host__ __device__ constexpr int fold_adj_min_blocks(int sums) { return sums <= 4 ? 6 : (sums <= 8 ? 5 : 4); }
 
-template <typename S, typename T, int M>
-__global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M))
-    fold_adj_kernel(const __grid_constant__ CUtensorMap tm_gt, const AdjProj *__restrict__ uproj,
-                    S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int U, int m, int Wb, T alpha, T beta,
-                    int *status, int PP) {
-    constexpr int VPT = FoldAdjShape<M>::VPT;
-    constexpr int TX = FoldAdjShape<M>::TX;
-    constexpr int TY = kAdjTY;
+template <typename S, typename T, int M, int ZS>
+__global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjShape<M>::MC))
+    fold_adj_kernel(const __grid_constant__ CUtensorMap tm_gt, const FoldAng *__restrict__ ang,
+                    S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int nz, int U, int U1, int m, T alpha,
+                    T beta, int *status, int PP, int vec) {
+    using Sh = FoldAdjShape<M>;
+    constexpr int TX = Sh::TX, TY = kAdjTY, SX = Sh::SX, NG = Sh::NG, MC = Sh::MC;
     constexpr int NST = kFoldAdjStages;
     constexpr int MS = fold_ms(M);
-    constexpr float kMag = 12582912.0f;
+    constexpr float kMag = 12582912.0f;  // 1.5 * 2^23: adding it rounds to an integer
     constexpr int kMagI = 0x4B400000;
+    constexpr bool PK = MC % 2 == 0;        // coefficient pairs
+    constexpr int NC = PK ? MC / 2 : MC;    // sums per voxel
+    constexpr int CH = MC % 4 == 0 ? 2 : (PK ? 1 : MC);  // sums per chunk of bin reads (16, 8 or 4 bytes)
+    using A = std::conditional_t<PK, unsigned long long, float>;
 
     extern __shared__ __align__(128) unsigned char fadj_smem_raw[];
     // round up to 128 B by pointer arithmetic on the __shared__ array, so the
     // compiler keeps addressing it as shared memory (LDS, not generic loads)
     unsigned char *smem_raw = fadj_smem_raw + ((128u - (smem_u32(fadj_smem_raw) & 127u)) & 127u);
-    const size_t row_bytes = ((size_t)Wb * MS * sizeof(T) + 127) & ~(size_t)127;
-    const size_t win_bytes = PP * row_bytes;
-    const size_t stage_bytes = win_bytes + 128 * ((PP * sizeof(FoldPrm) + 127) / 128);
+    constexpr int WIN = Sh::WIN;  // floats of one slice's window of one angle
+    const int win_bytes = PP * ZS * WIN * (int)sizeof(T);
+    const int stage_bytes = win_bytes + 128 * ((PP * (int)sizeof(FoldPrm) + 127) / 128);
     __shared__ __align__(8) uint64_t full[NST];
-    auto win_s = [&](int st, int p) { return reinterpret_cast<T *>(smem_raw + st * stage_bytes + p * row_bytes); };
+    auto win_s = [&](int st, int p) { return reinterpret_cast<T *>(smem_raw + st * stage_bytes) + p * ZS * WIN; };
     auto prm_s = [&](int st) { return reinterpret_cast<FoldPrm *>(smem_raw + st * stage_bytes + win_bytes); };
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ntx = (nx + TX - 1) / TX;
     const int x0 = (blockIdx.x % ntx) * TX, y0 = (blockIdx.x / ntx) * TY;
-    const int z = blockIdx.y;
-    const int xo = x0 + TX / 2, yo = y0 + TY / 2;
-    constexpr bool PAIRED = FoldAdjShape<M>::PAIRED;
-    const int tx = PAIRED ? (tid & 15) : (tid & 7), ty = PAIRED ? (tid >> 4) : (tid >> 3);
-    const int dx0 = x0 + tx - xo, dy = (PAIRED ? y0 + 2 * ty : y0 + ty) - yo;
-    const int nkb = (U + PP - 1) / PP;
+    const int z0 = blockIdx.y * ZS;
+    // patch of this thread: a warp covers 8 x 4 patches, a quarter of it 4 x 2
+    const int vw = NG == 1 ? warp : (warp & 1), cg = NG == 1 ? 0 : (warp >> 1);
+    const int px = (lane & 3) + 4 * ((lane >> 3) & 1) + (NG == 1 ? 8 * (vw & 1) : 0);
+    const int py = ((lane >> 2) & 1) + 2 * (lane >> 4) + 4 * (NG == 1 ? vw >> 1 : vw);
+    const int dx = 2 * px, dy = 2 * py;
+    // blocks of PP angles: those with cos >= 0 (the first U1), then the others
+    const int nk1 = (U1 + PP - 1) / PP, nkb = nk1 + (U - U1 + PP - 1) / PP;
+    auto first = [&](int kb) { return kb < nk1 ? kb * PP : U1 + (kb - nk1) * PP; };
+    auto past = [&](int kb) { return kb < nk1 ? U1 : U; };
 
+    // One lane per angle: window and constants, TMA copies.
     auto issue = [&](int st, int kb) {
-        int wb0 = 0, row = 0;
+        int wb0 = 0, aa = 0;
         if (lane < PP) {
-            const int a = kb * PP + lane;
-            const int aa = a < U ? a : U - 1;
-            const AdjProj pj = uproj[aa];
-            const double posO = xo * pj.c + yo * pj.s + pj.C0;
-            const double emin = posO + fmin((-TX / 2) * pj.c, (TX / 2 - 1) * pj.c) +
-                                fmin((-TY / 2) * pj.s, (TY / 2 - 1) * pj.s);
-            wb0 = (int)floor(emin) - 1;
-            const double rel = posO - wb0;
-            const double ri = floor(rel);
+            aa = min(first(kb) + lane, past(kb) - 1);
+            const FoldAng pj = ang[aa];
             FoldPrm pr;
-            pr.c = (float)pj.c;
-            pr.s = (float)pj.s;
-            pr.c8 = (float)(8.0 * pj.c);
-            pr.qb = (float)(rel - ri) - 0.5f;
-            pr.inv_c2 = (float)(pj.inv_c * pj.inv_c);
-            pr.e0 = (float)(pj.inv_c - 0.5 * pj.inv_c * pj.inv_c);
-            pr.idx_base = (int)ri - kMagI;
-            pr.c16 = (float)(16.0 * pj.c);
+            pr.c = pj.cf;
+            pr.s = pj.sf;
+            pr.c16 = pj.c16;
+            pr.e0 = pj.e0;
+            pr.inv_c2 = pj.inv_c2;
+            const int yo = y0 + TY / 2;
+#pragma unroll
+            for (int k = 0; k < TX / SX; ++k) {
+                const int xo = x0 + k * SX + SX / 2;
+                const double posO = xo * pj.c + yo * pj.s + pj.C0, fl = floor(posO);
+                if (k == 0)  // the tile's lowest position, less a bin for rounding
+                    wb0 = (int)fl - 1 + (int)floorf(fminf((-SX / 2) * pj.cf, (TX - 1 - SX / 2) * pj.cf) +
+                                                    fminf((-TY / 2) * pj.sf, (TY / 2 - 1) * pj.sf));
+                pr.sub[k].qb = (float)(posO - fl) - 0.5f;
+                pr.sub[k].idx = (int)fl - wb0 - kMagI;
+            }
             prm_s(st)[lane] = pr;
-            row = z * U + aa;
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive_expect_tx(&full[st], (unsigned)(PP * Wb * MS * sizeof(T)));
+        if (lane == 0) mbar_arrive_expect_tx(&full[st], (unsigned)win_bytes);
         __syncwarp();
-        if (lane < PP) tma_load_3d(win_s(st, lane), &tm_gt, 0, wb0, row, &full[st]);
+        if (lane < PP) {
+#pragma unroll
+            for (int k = 0; k < ZS; ++k)  // (slices beyond the volume: the last one again, not stored)
+                for (int i = 0; i < Sh::NBOX; ++i)
+                    tma_load_2d(win_s(st, lane) + k * WIN + i * Sh::BOX, &tm_gt, wb0 * MS + i * Sh::BOX,
+                                min(z0 + k, nz - 1) * U + aa, &full[st]);
+        }
         if (lane != 0) mbar_arrive(&full[st]);
     };
 
@@ -759,84 +811,138 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M))
     if (warp == 0)
         for (int s = 0; s < NST && s < nkb; ++s) issue(s, s);
 
-    T acc[VPT][M];
+    // sums of voxel (x + i, y + j) at [j][i]; for the angles with c < 0 the
+    // columns are swapped, so that column 0 is always the lower one on the detector
+    A acc[ZS][2][2][NC];
 #pragma unroll
-    for (int v = 0; v < VPT; ++v)
+    for (int k = 0; k < ZS; ++k)
 #pragma unroll
-        for (int j = 0; j < M; ++j) acc[v][j] = T(0);
+        for (int v = 0; v < 4; ++v)
+#pragma unroll
+            for (int q = 0; q < NC; ++q) acc[k][v >> 1][v & 1][q] = 0;
+    // x of the lower (dA) and the upper column from the subtile's middle, and the
+    // half of a 32-wide subtile that they lie in
+    const int sub = dx / SX, sx = dx - sub * SX;
+    float dA = (float)((sx & 15) - SX / 2), dB = dA + 1.0f;
+    const bool far = sx >= 16;
+    const float dyf = (float)(dy - TY / 2);
+    auto flip = [&]() {
+        const float t = dA;
+        dA = dB;
+        dB = t;
+#pragma unroll
+        for (int j = 0; j < 2 * ZS; ++j)
+#pragma unroll
+            for (int q = 0; q < NC; ++q) {
+                const A t = acc[j >> 1][j & 1][0][q];
+                acc[j >> 1][j & 1][0][q] = acc[j >> 1][j & 1][1][q];
+                acc[j >> 1][j & 1][1][q] = t;
+            }
+    };
+    auto dup = [](float w) -> A {
+        if constexpr (PK) return pack_f2(w, w);
+        else return w;
+    };
+    auto mad = [](A w, A b, A r) {
+        if constexpr (PK) return fma_f2(w, b, r);
+        else return fmaf(w, b, r);
+    };
 
-    const float dxf = (float)dx0, dyf = (float)dy;
     for (int kb = 0; kb < nkb; ++kb) {
         const int st = kb % NST;
         const bool bad = !mbar_wait_bounded(&full[st], (unsigned)((kb / NST) & 1), status, 2000000000ull);
-        if (!bad) {
-            const FoldPrm *prm = prm_s(st);
-            const int np = min(PP, U - kb * PP);
-            for (int p = 0; p < np; ++p) {
-                const FoldPrm a = prm[p];
-                const T *w = win_s(st, p);
-                float q = fmaf(dyf, a.s, fmaf(dxf, a.c, a.qb));
-                // Pairs need the two rows' taps within three bins: |qB - qA| < 1.
-                // With |sin| <= 1 - 1e-5 and |q| < 64 (rounding of qA + sin below
-                // 4e-6) the rounded bin indices differ by at most one; angles
-                // closer to |sin| = 1 (a warp-uniform test) use the per-voxel path.
-                if (PAIRED && fabsf(a.s) <= 0.99999f) {
-#pragma unroll
-                    for (int v = 0; v < VPT / 2; ++v) {
-                        // rows y (A) and y + 1 (B) of column v
-                        const float qA = q, qB = q + a.s;
-                        const float tA = qA + kMag, tB = qB + kMag;
-                        const float dA = qA - (tA - kMag), dB = qB - (tB - kMag);
-                        const int iA = __float_as_int(tA) + a.idx_base, iB = __float_as_int(tB) + a.idx_base;
-                        const float w0A = fmaxf(0.0f, fmaf(-dA, a.inv_c2, a.e0));
-                        const float w1A = fmaxf(0.0f, fmaf(dA, a.inv_c2, a.e0));
-                        const float w0B = fmaxf(0.0f, fmaf(-dB, a.inv_c2, a.e0));
-                        const float w1B = fmaxf(0.0f, fmaf(dB, a.inv_c2, a.e0));
-                        {
-                            // taps iA, iA+1 and iB, iB+1 within bins b, b+1, b+2: each
-                            // voxel's weights on the three bins (one of them an exact 0)
-                            const int b = min(iA, iB);
-                            const bool lA = iA == b, lB = iB == b;
-                            const float oA0 = lA ? w0A : 0.0f, oA1 = lA ? w1A : w0A, oA2 = lA ? 0.0f : w1A;
-                            const float oB0 = lB ? w0B : 0.0f, oB1 = lB ? w1B : w0B, oB2 = lB ? 0.0f : w1B;
-                            const T *r0 = w + b * MS;
-                            constexpr int CH = (M % 4) == 0 ? 4 : M;  // coefficients per chunk
-#pragma unroll
-                            for (int c0 = 0; c0 < M; c0 += CH) {
-                                T b0[CH], b1[CH], b2[CH];
-                                load_vec<T, CH>(r0 + c0, b0);
-                                load_vec<T, CH>(r0 + MS + c0, b1);
-                                load_vec<T, CH>(r0 + 2 * MS + c0, b2);
-#pragma unroll
-                                for (int j = 0; j < CH; ++j) {
-                                    T &ra = acc[2 * v][c0 + j];
-                                    ra = fmaf(oA2, b2[j], fmaf(oA1, b1[j], fmaf(oA0, b0[j], ra)));
-                                    T &rb = acc[2 * v + 1][c0 + j];
-                                    rb = fmaf(oB2, b2[j], fmaf(oB1, b1[j], fmaf(oB0, b0[j], rb)));
-                                }
-                            }
-                        }
-                        q += a.c16;
-                    }
-                    continue;
+        const FoldPrm *prm = prm_s(st);
+        const int np = bad ? 0 : min(PP, past(kb) - first(kb));
+        if (kb == nk1) flip();
+        for (int p = 0; p < np; ++p) {
+            const float4 h = *reinterpret_cast<const float4 *>(prm + p);  // c, s, c16, e0
+            const float ac = h.x, as = h.y, ic2 = prm[p].inv_c2, qb = prm[p].sub[sub].qb;
+            const int idx = prm[p].sub[sub].idx;
+            // positions of the patch's voxels: lower and upper column, two rows
+            float qA = fmaf(dyf, as, fmaf(dA, ac, qb)), qB = fmaf(dyf, as, fmaf(dB, ac, qb));
+            float qC, qD;
+            if constexpr (Sh::STEP) {
+                if (SX == 32) {
+                    const float e = far ? h.z : 0.0f;
+                    qA += e;
+                    qB += e;
                 }
-                // one voxel at a time: voxel v at q (+ sin for the second row of a pair)
+                qC = qA + as;
+                qD = qB + as;
+            } else {
+                qC = fmaf(dyf + 1.0f, as, fmaf(dA, ac, qb));
+                qD = fmaf(dyf + 1.0f, as, fmaf(dB, ac, qb));
+            }
+            // a voxel's lower bin and the weights of its two bins
+            auto taps = [&](float q, float &w0, float &w1) {
+                const float t = q + kMag, d = q - (t - kMag);
+                w0 = fmaxf(0.0f, fmaf(-d, ic2, h.w));
+                w1 = fmaxf(0.0f, fmaf(d, ic2, h.w));
+                return __float_as_int(t) + idx;
+            };
+            if (fabsf(ac) > 0.99999f || fabsf(as) > 0.99999f) {
+                // close to an axis: each voxel's two bins by themselves
+                const float qv[4] = {qA, qB, qC, qD};
 #pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    const float qv = (PAIRED && (v & 1)) ? q + a.s : q;
-                    const float t = qv + kMag;
-                    const float fl = t - kMag;
-                    const float d = qv - fl;
-                    const int idx = __float_as_int(t) + a.idx_base;
-                    const float w0 = fmaxf(0.0f, fmaf(-d, a.inv_c2, a.e0));
-                    const float w1 = fmaxf(0.0f, fmaf(d, a.inv_c2, a.e0));
-                    T t0[M], t1[M];
-                    load_vec<T, M>(w + idx * MS, t0);
-                    load_vec<T, M>(w + (idx + 1) * MS, t1);
+                for (int v = 0; v < 4; ++v) {
+                    float w0, w1;
+                    const T *r0 = win_s(st, p) + taps(qv[v], w0, w1) * MS + cg * MC;
+                    const A p0 = dup(w0), p1 = dup(w1);
 #pragma unroll
-                    for (int j = 0; j < M; ++j) acc[v][j] = fmaf(w1, t1[j], fmaf(w0, t0[j], acc[v][j]));
-                    if (!PAIRED) q += a.c8;
-                    else if (v & 1) q += a.c16;
+                    for (int k = 0; k < ZS; ++k)
+#pragma unroll
+                        for (int q = 0; q < NC; ++q) {
+                            const A *r = reinterpret_cast<const A *>(r0 + k * WIN) + q;
+                            A &t = acc[k][v >> 1][v & 1][q];
+                            t = mad(p1, *reinterpret_cast<const A *>(r0 + k * WIN + MS + q * (PK ? 2 : 1)), mad(p0, *r, t));
+                        }
+                }
+                continue;
+            }
+            float w0, w1;
+            const int b0 = taps(qA, w0, w1);
+            const T *w = win_s(st, p) + b0 * MS + cg * MC;
+            const A p00 = dup(w0), p01 = dup(w1);
+            A p1[3], p2[3], p3[3];
+            // weights on three candidate bins, the first of them lim - 1 bins on
+            auto three = [&](float q, int lim, A (&o)[3]) {
+                const bool on = taps(q, w0, w1) - b0 >= lim;
+                o[0] = dup(on ? 0.0f : w0);
+                o[1] = dup(on ? w0 : w1);
+                o[2] = dup(on ? w1 : 0.0f);
+            };
+            three(qB, 1, p1);
+            three(qC, 1, p2);
+            three(qD, 2, p3);
+#pragma unroll
+            for (int k = 0; k < ZS; ++k) {
+                const T *ws = w + k * WIN;
+#pragma unroll
+                for (int q0 = 0; q0 < NC; q0 += CH) {
+                    A bin[4][CH];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const T *r = ws + i * MS + q0 * (PK ? 2 : 1);
+                        if constexpr (PK && CH == 2) {
+                            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(r);
+                            bin[i][0] = v.x;
+                            bin[i][1] = v.y;
+                        } else if constexpr (PK) {
+                            bin[i][0] = *reinterpret_cast<const unsigned long long *>(r);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < CH; ++q) bin[i][q] = r[q];
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < CH; ++q) {
+                        A &r0 = acc[k][0][0][q0 + q], &r1 = acc[k][0][1][q0 + q], &r2 = acc[k][1][0][q0 + q],
+                          &r3 = acc[k][1][1][q0 + q];
+                        r0 = mad(p01, bin[1][q], mad(p00, bin[0][q], r0));
+                        r1 = mad(p1[2], bin[2][q], mad(p1[1], bin[1][q], mad(p1[0], bin[0][q], r1)));
+                        r2 = mad(p2[2], bin[2][q], mad(p2[1], bin[1][q], mad(p2[0], bin[0][q], r2)));
+                        r3 = mad(p3[2], bin[3][q], mad(p3[1], bin[2][q], mad(p3[0], bin[1][q], r3)));
+                    }
                 }
             }
         }
@@ -846,26 +952,53 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M))
                     mbar_wait_bounded(&full[s % NST], (unsigned)((s / NST) & 1), status, 100000000ull);
             return;
         }
-        if (warp == 0 && kb + NST < nkb) issue(st, kb + NST);
+        // (the warps refill in turn: the others are already at the next stage)
+        if (warp == (kb & 3) && kb + NST < nkb) issue(st, kb + NST);
     }
+    if (nk1 < nkb) flip();
 
 #pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-        const int x = PAIRED ? x0 + tx + 16 * (v >> 1) : x0 + tx + 8 * v;
-        const int y = PAIRED ? y0 + 2 * ty + (v & 1) : y0 + ty;
-        if (x >= nx || y >= ny) continue;
-        const size_t base = (((size_t)z * ny + y) * nx + x) * m;
+    for (int v = 0; v < 4 * ZS; ++v) {
+        const int x = x0 + dx + (v & 1), y = y0 + dy + ((v >> 1) & 1), z = z0 + (v >> 2);
+        if (x >= nx || y >= ny || z >= nz) continue;
+        const size_t base = (((size_t)z * ny + y) * nx + x) * m + cg * MC;
+        float r[MC];
+        if constexpr (PK) {
 #pragma unroll
-        for (int j = 0; j < M; ++j)
-            if (j < m) {
+            for (int q = 0; q < NC; ++q) unpack_f2(acc[v >> 2][(v >> 1) & 1][v & 1][q], r[2 * q], r[2 * q + 1]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < NC; ++q) r[q] = acc[v >> 2][(v >> 1) & 1][v & 1][q];
+        }
+#pragma unroll
+        for (int j = 0; j < MC; ++j) r[j] *= alpha;
+        if constexpr (sizeof(S) == 4 && MC % 4 == 0) {
+            if (vec) {  // rows of whole 16-byte vectors
+                float4 *d = reinterpret_cast<float4 *>((u_c ? u_c : (T *)u_s) + base);
+#pragma unroll
+                for (int q = 0; q < MC / 4; ++q) {
+                    float4 o = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                    if (beta != T(0)) {
+                        const float4 b = d[q];
+                        o.x += beta * b.x;
+                        o.y += beta * b.y;
+                        o.z += beta * b.z;
+                        o.w += beta * b.w;
+                    }
+                    d[q] = o;
+                }
+                continue;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < MC; ++j)
+            if (cg * MC + j < m) {
                 if (u_c) {
-                    T r = alpha * acc[v][j];
-                    if (beta != T(0)) r += beta * u_c[base + j];
-                    u_c[base + j] = r;
+                    if (beta != T(0)) r[j] += beta * u_c[base + j];
+                    u_c[base + j] = r[j];
                 } else {
-                    T r = alpha * acc[v][j];
-                    if (beta != T(0)) r += beta * ldc<T>(u_s + base + j);
-                    stc<T>(u_s + base + j, r);
+                    if (beta != T(0)) r[j] += beta * ldc<T>(u_s + base + j);
+                    stc<T>(u_s + base + j, r[j]);
                 }
             }
     }
@@ -874,13 +1007,6 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M))
 // ===========================================================================
 // Host launchers
 // ===========================================================================
-inline int fold_adj_wb(int M) {
-    const int VPT = (M <= 8) ? 4 : ((M <= 16) ? 2 : 1);
-    const int TX = 8 * VPT;
-    const double ext = std::sqrt((double)(TX - 1) * (TX - 1) + (double)(kAdjTY - 1) * (kAdjTY - 1));
-    return (int)std::ceil(ext) + 6;
-}
-
 template <typename S, typename T, int M>
 dr_status fold_fwd_launch_t(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                             cudaStream_t st) {
@@ -1080,29 +1206,31 @@ template <typename S, typename T, int M>
 dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool u_calc, cudaStream_t st, void *gt) {
     constexpr int MS = fold_ms(M);
     if (!gt) gt = P->d_gt;
-    const int Wb = fold_adj_wb(M);
     CUtensorMap tm{};
-    const uint64_t dims[3] = {(uint64_t)MS, (uint64_t)P->ns, (uint64_t)P->nz * P->fold_U};
-    const uint64_t strides[2] = {(uint64_t)MS * sizeof(T), (uint64_t)P->ns * MS * sizeof(T)};
-    const uint32_t box[3] = {(uint32_t)MS, (uint32_t)Wb, 1};
-    if (!encode_tensor_map(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, gt, dims, strides, box))
+    if (!encode_tensor_map_2d(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, gt, (uint64_t)P->ns * MS, (uint64_t)P->nz * P->fold_U,
+                              (uint64_t)P->ns * MS * sizeof(T), (uint32_t)FoldAdjShape<M>::BOX, 1))
         return fail(DR_ECUDA, "fold adj: tensor map encode failed");
+    constexpr int TX = FoldAdjShape<M>::TX, ZMAX = FoldAdjShape<M>::ZS;
+    const int ntx = (P->nx + TX - 1) / TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
+    // several slices per thread where that leaves every SM its resident CTAs
+    const int zs = ZMAX > 1 && (long long)ntx * nty * ((P->nz + ZMAX - 1) / ZMAX) >=
+                                   (long long)P->num_sms * fold_adj_min_blocks(ZMAX * FoldAdjShape<M>::MC)
+                       ? ZMAX : 1;
     // angles per pipeline stage: fewer shrink the windows' shared memory so that
     // more CTAs fit on an SM (the angles are summed in the same order)
-    const int pp = std::max(1, std::min(32, P->fold_adj_pp));
-    const size_t row_bytes = ((size_t)Wb * MS * sizeof(T) + 127) & ~(size_t)127;
-    const size_t stage = pp * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128);
+    constexpr int row_bytes = FoldAdjShape<M>::WIN * (int)sizeof(T);
+    const int pp = std::max(1, std::min(std::min(32, P->fold_adj_pp), kFoldAdjWin / (zs * row_bytes)));
+    const size_t stage = (size_t)pp * zs * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128);
     const size_t smem = stage * kFoldAdjStages + 128;
-    auto kern = fold_adj_kernel<S, T, M>;
+    auto kern = zs > 1 ? fold_adj_kernel<S, T, M, ZMAX> : fold_adj_kernel<S, T, M, 1>;
     {
         dr_status s = allow_dynamic_smem((const void *)kern, smem);
         if (s != DR_OK) return s;
     }
-    constexpr int TX = FoldAdjShape<M>::TX;
-    const int ntx = (P->nx + TX - 1) / TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
-    dim3 grid(ntx * nty, P->nz);
-    kern<<<grid, kAdjThreads, smem, st>>>(tm, P->d_fold_adj, u_calc ? nullptr : (S *)u, u_calc ? (T *)u : nullptr,
-                                          P->nx, P->ny, P->fold_U, P->m, Wb, (T)alpha, (T)beta, P->d_status, pp);
+    dim3 grid(ntx * nty, (P->nz + zs - 1) / zs);
+    kern<<<grid, kAdjThreads, smem, st>>>(tm, P->d_fold_ang, u_calc ? nullptr : (S *)u, u_calc ? (T *)u : nullptr,
+                                          P->nx, P->ny, P->nz, P->fold_U, P->fold_U1, P->m, (T)alpha, (T)beta, P->d_status, pp,
+                                          P->m == M && ((uintptr_t)u & 15u) == 0);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "fold_adj_kernel launch");
 }

@@ -386,7 +386,7 @@ static dr_status build_tables(dr_plan *P) {
         int maxg = 0;
         for (int a = 0; a < U; ++a) maxg = std::max(maxg, start[a + 1] - start[a]);
         std::vector<FwdProj> ufw(U);
-        std::vector<AdjProj> uad(U);
+        std::vector<FoldAng> uad(U);
         std::vector<int> ub0, ub1;
         for (int a = 0; a < U; ++a) {
             const double c = std::cos(rep[a]), s = std::sin(rep[a]);
@@ -401,7 +401,9 @@ static dr_status build_tables(dr_plan *P) {
             f.A_fx = std::llround(f.A * two32); f.B_fx = std::llround(f.B * two32); f.C_fx = std::llround(f.C * two32);
             f.Af = (float)f.A; f.Bf = (float)f.B; f.Cf = (float)f.C; f.scale = (float)f.scale_d;
             ufw[a] = f;
-            uad[a] = make_adj(c, s, -hx * c - hy * s + hs);
+            const AdjProj j = make_adj(c, s, -hx * c - hy * s + hs);
+            uad[a] = FoldAng{j.c, j.s, j.C0, (float)j.c, (float)j.s, (float)(16.0 * j.c),
+                             (float)std::fma(-0.5 * j.inv_c, j.inv_c, j.inv_c), (float)(j.inv_c * j.inv_c), 0.0f};
         }
         // forward work lists over unique angles
         const int M = P->M;
@@ -422,6 +424,8 @@ static dr_status build_tables(dr_plan *P) {
             for (size_t i = 0; i < grp->size(); i += Pf)
                 for (int q = 0; q < Pf; ++q) fb.push_back(i + q < grp->size() ? (*grp)[i + q] : -1);
         P->fold_U = U;
+        P->fold_U1 = 0;
+        while (P->fold_U1 < U && uad[P->fold_U1].c >= 0.0) ++P->fold_U1;
         P->fold_maxgrp = maxg;
         P->fold_P = Pf;
         P->fold_R = std::max(R, 1);  // lines of one strip buffer that fit the shared-memory strip budget
@@ -432,13 +436,13 @@ static dr_status build_tables(dr_plan *P) {
         P->fold_nchunk = nchunk;
         P->n_fold_blocks = (int)(fb.size() / Pf);
         DR_CUDA_TRY(cudaMalloc(&P->d_fold_fwd, sizeof(FwdProj) * U));
-        DR_CUDA_TRY(cudaMalloc(&P->d_fold_adj, sizeof(AdjProj) * U));
+        DR_CUDA_TRY(cudaMalloc(&P->d_fold_ang, sizeof(FoldAng) * U));
         DR_CUDA_TRY(cudaMalloc(&P->d_fold_start, sizeof(int) * (U + 1)));
         DR_CUDA_TRY(cudaMalloc(&P->d_fold_member, sizeof(int) * K));
         DR_CUDA_TRY(cudaMalloc(&P->d_fold_blocks, sizeof(int) * std::max<size_t>(fb.size(), 1)));
-        bytes += (sizeof(FwdProj) + sizeof(AdjProj) + sizeof(int)) * U + sizeof(int) * (K + 1 + fb.size());
+        bytes += (sizeof(FwdProj) + sizeof(FoldAng) + sizeof(int)) * U + sizeof(int) * (K + 1 + fb.size());
         DR_CUDA_TRY(cudaMemcpy(P->d_fold_fwd, ufw.data(), sizeof(FwdProj) * U, cudaMemcpyHostToDevice));
-        DR_CUDA_TRY(cudaMemcpy(P->d_fold_adj, uad.data(), sizeof(AdjProj) * U, cudaMemcpyHostToDevice));
+        DR_CUDA_TRY(cudaMemcpy(P->d_fold_ang, uad.data(), sizeof(FoldAng) * U, cudaMemcpyHostToDevice));
         DR_CUDA_TRY(cudaMemcpy(P->d_fold_start, start.data(), sizeof(int) * (U + 1), cudaMemcpyHostToDevice));
         DR_CUDA_TRY(cudaMemcpy(P->d_fold_member, member.data(), sizeof(int) * K, cudaMemcpyHostToDevice));
         if (!fb.empty())
@@ -624,7 +628,7 @@ dr_status dr_plan_destroy(dr_plan *P) {
     free_workspace(P);
     void *ptrs[] = {P->d_fwd,        P->d_adj,       P->d_PhiP,       P->d_fwd_blocks,  P->d_PhiF,
                     P->d_dPhiF,      P->d_G,         P->d_Lt,         P->d_partials,    P->d_counters,
-                    P->d_scal,       P->d_status,    P->d_fold_fwd,   P->d_fold_adj,    P->d_fold_start,
+                    P->d_scal,       P->d_status,    P->d_fold_fwd,   P->d_fold_ang,    P->d_fold_start,
                     P->d_fold_member, P->d_fold_blocks, P->d_gt, P->d_fbp_taps, P->d_fbp_phi, P->d_fbp_q,
                     P->d_fbp_u, P->d_ru_split, P->d_fold_gram};
     for (void *p : ptrs)
