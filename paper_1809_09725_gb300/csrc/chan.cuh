@@ -33,11 +33,15 @@ struct StaticOut {
 // forward variant of automatic operator calls and Chambolle-Pock, where the
 // autotuner found it faster (reported as the fold in two kernels)
 constexpr int kVarChan = 3;
+// the same kernel in the summation order, and with the line chunks, of the fold
+// in two kernels, whose values it then gives bit for bit (ADMM)
+constexpr int kVarChanEO = 4;
+inline int fold2_chunks(const dr_plan *P) { return P->split_off ? 1 : (P->fold2_split > 1 ? P->fold2_split : 1); }
 constexpr int kChanWarps = 16;  // compute warps per CTA, at most (8: two CTAs per SM); one more copies
 constexpr int kChanSlots = 8;   // line buffers in flight, at most
 constexpr int kChanBox = 8;     // pixels per TMA box
 // bytes of line buffers of a CTA of nw compute warps
-__host__ __device__ constexpr int chan_ring(int nw) { return (nw == 8 ? 108 : 220) * 1024; }
+__host__ __device__ constexpr int chan_ring(int nw) { return (nw == 8 ? 108 : 216) * 1024; }
 constexpr int kChanMin = 32;                // least channels (nz times m rounded up to 4) that the kernels take
 constexpr size_t kChanScratchMax = size_t(1) << 30;  // packed volume held at a time
 // rays per warp: 64 sums per lane at V = 2 and 4, 32 at V = 1
@@ -45,9 +49,10 @@ __host__ __device__ constexpr int chan_rw(int V) { return V == 4 ? 16 : 32; }
 __host__ __device__ constexpr int chan_boxes(int px) { return (px + kChanBox - 1) / kChanBox; }
 
 dr_status chan_setup(dr_plan *P, const std::vector<FwdProj> &fw);
-bool chan_fwd_ready(dr_plan *P, cudaStream_t st);
+bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st);
 // static transforms of u (bf: stored bf16, else float); chan_fwd_ready must hold
-dr_status chan_static(dr_plan *P, const void *u, bool bf, cudaStream_t st, StaticOut &rs);
+// (eo: each sample's even pixel first, the order of the thread-per-ray kernels)
+dr_status chan_static(dr_plan *P, const void *u, bool bf, bool eo, int nsplit, cudaStream_t st, StaticOut &rs);
 void chan_free(dr_plan *P);
 
 inline RowMap slice_rows(size_t rows_per_slice, int ms) { return RowMap{1, ms, ms, rows_per_slice * ms}; }

@@ -23,6 +23,12 @@
 // rate).  Tried and slower: packed multiply-adds (0.405 ms: the copies that
 // pair the weights), a real branch instead of the predicated read (0.387 ms),
 // two lines at a time (0.390 ms with 16 warps, against 0.396 ms).
+//
+// EO: the same march in the order of the thread-per-ray kernels (a sample's even
+// pixel is added before its odd one): the even and the odd pixel keep their own
+// registers, and the lanes work out weights and steps of a line's rays side by
+// side.  Bit for bit the fold in two kernels, so ADMM can run on it; 0.44 ms
+// (three line chunks) and 8.5 ms on the two volumes above.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -68,6 +74,47 @@ __device__ __forceinline__ void chan_advance(unsigned &frac, unsigned a, uint32_
     frac = f;
 }
 
+// One step along a line in even / odd order: where bit K of the mask is set,
+// a += step and v = [a].
+template <int V, int K>
+__device__ __forceinline__ void chan_step(unsigned mask, uint32_t &a, int step, float (&v)[V]) {
+    if constexpr (V == 1)
+        asm volatile(
+            "{\n\t.reg .pred c;\n\t.reg .u32 t;\n\tand.b32 t, %2, %4;\n\tsetp.ne.u32 c, t, 0;\n\t"
+            "@c add.u32 %0, %0, %3;\n\t@c ld.shared.f32 %1, [%0];\n\t}"
+            : "+r"(a), "+f"(v[0])
+            : "r"(mask), "r"(step), "n"(1u << K));
+    else if constexpr (V == 2)
+        asm volatile(
+            "{\n\t.reg .pred c;\n\t.reg .u32 t;\n\tand.b32 t, %3, %5;\n\tsetp.ne.u32 c, t, 0;\n\t"
+            "@c add.u32 %0, %0, %4;\n\t@c ld.shared.v2.f32 {%1, %2}, [%0];\n\t}"
+            : "+r"(a), "+f"(v[0]), "+f"(v[1])
+            : "r"(mask), "r"(step), "n"(1u << K));
+    else
+        asm volatile(
+            "{\n\t.reg .pred c;\n\t.reg .u32 t;\n\tand.b32 t, %5, %7;\n\tsetp.ne.u32 c, t, 0;\n\t"
+            "@c add.u32 %0, %0, %6;\n\t@c ld.shared.v4.f32 {%1, %2, %3, %4}, [%0];\n\t}"
+            : "+r"(a), "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3])
+            : "r"(mask), "r"(step), "n"(1u << K));
+}
+// Rays K, K + 1, .. of a line: the even pixel of each in e, the odd one in o.
+template <int V, int RW, int K>
+__device__ __forceinline__ void chan_line(unsigned me, unsigned mo, uint32_t &pe, uint32_t &po, const float4 *rec,
+                                          float4 &w, float (&e)[V], float (&o)[V], float (&acc)[RW][V]) {
+    if constexpr (K < RW) {
+        if constexpr (K > 0) {
+            chan_step<V, K>(me, pe, 2 * 128 * V, e);
+            chan_step<V, K>(mo, po, 2 * 128 * V, o);
+        }
+        if constexpr ((K & 3) == 0) w = rec[K >> 2];
+        // (a weight is a multiple of 2^-23: the other one is exactly 1 less it)
+        const float we = (K & 3) == 0 ? w.x : (K & 3) == 1 ? w.y : (K & 3) == 2 ? w.z : w.w, wo = 1.0f - we;
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[K][v] = fmaf(wo, o[v], fmaf(we, e[v], acc[K][v]));
+        chan_line<V, RW, K + 1>(me, mo, pe, po, rec, w, e, o, acc);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // uc[block][pixel][C] <- u[z][pixel][m]: channel zi ms + j of block c is
 // coefficient j of slice c spb + zi (zero for j >= m and beyond the volume).
@@ -110,7 +157,7 @@ struct ChanFwdArgs {
     int n, g, nx, ny, ns, nz, c0, ms, spb, ring_bytes;
 };
 
-template <int V, int RW, int NW>
+template <int V, int RW, int NW, bool EO>
 __global__ void __launch_bounds__(32 * (NW + 1), NW == 8 ? 2 : 1)
     chan_fwd_kernel(const __grid_constant__ CUtensorMap tm_rows, const __grid_constant__ CUtensorMap tm_cols,
                     const __grid_constant__ ChanFwdArgs P) {
@@ -122,6 +169,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), NW == 8 ? 2 : 1)
     __shared__ int base_s[kChanSlots];  // byte offset of pixel 0 of a buffered line (of its band's first pixel less s0)
     __shared__ long long x_s[NW], e_s[NW], b_s[NW];  // first / last ray, step per line
     __shared__ int lo_s[NW], hi_s[NW];
+    __shared__ __align__(16) float rec_s[EO ? NW : 1][2][32];  // weights of the even pixel
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cb = blockIdx.y, chunk = blockIdx.z;
@@ -296,9 +344,41 @@ __global__ void __launch_bounds__(32 * (NW + 1), NW == 8 ? 2 : 1)
     const uint32_t mine = smem_u32(ring) + lane * (4 * V);
     int slot = 0;
     unsigned phase = 0;
+    // even / odd order: the lanes work out the rays of one line (RW = 32) or two
+    // (RW = 16) side by side: weights to shared memory, and in two masks the rays
+    // at which the even and the odd pixel change
+    constexpr int NL = 32 / RW;
+    const int rq = lane % RW;
+    const long long roff = (lane / RW) * bstep + rq * ((1ll << 32) + afrac);
+    unsigned me = 0, mo = 0;
+    int eb = 0, ob = 0, buf = 0;
     for (int r = rlo; r <= rhi; ++r) {
+        const int hl = EO ? (r - rlo) % NL : 0;
+        if (EO && hl == 0) {
+            const long long xr = x + roff;
+            const int i0 = (int)(xr >> 32);
+            const float w = __uint_as_float(__funnelshift_r((unsigned)xr, 0x7Fu, 9)) - 1.0f, w1m = 1.0f - w;
+            buf ^= 1;
+            rec_s[EO ? warp : 0][buf][lane] = (i0 & 1) ? w : w1m;
+            eb = (i0 + 1) & ~1;
+            ob = i0 | 1;
+            const int pe = __shfl_up_sync(0xffffffffu, eb, 1), po = __shfl_up_sync(0xffffffffu, ob, 1);
+            me = __ballot_sync(0xffffffffu, eb != pe);
+            mo = __ballot_sync(0xffffffffu, ob != po);
+            __syncwarp();
+        }
         if (!mbar_wait_bounded_any(&full[slot], phase, P.status, 2000000000ull)) return;
-        if (r >= wlo && r <= whi) {
+        if (EO && r >= wlo && r <= whi) {
+            uint32_t pe = mine + base_s[slot] + __shfl_sync(0xffffffffu, eb, hl * RW) * PXB;
+            uint32_t po = mine + base_s[slot] + __shfl_sync(0xffffffffu, ob, hl * RW) * PXB;
+            float e[V], o[V];
+            float4 w;
+            chan_ld<V>(pe, e);
+            chan_ld<V>(po, o);
+            chan_line<V, RW, 0>(NL > 1 ? me >> (hl * RW) : me, NL > 1 ? mo >> (hl * RW) : mo, pe, po,
+                                reinterpret_cast<const float4 *>(&rec_s[EO ? warp : 0][buf][hl * RW]), w, e, o, acc);
+        }
+        if (!EO && r >= wlo && r <= whi) {
             // one line: the two pixels of a ray in t[q & 1] and t[(q + 1) & 1]
             uint32_t p = mine + base_s[slot] + (int)(x >> 32) * PXB;
             unsigned frac = (unsigned)x;
@@ -554,11 +634,11 @@ static bool chan_alloc(void **p, size_t &held, size_t bytes, cudaStream_t st) {
     return true;
 }
 
-bool chan_fwd_ready(dr_plan *P, cudaStream_t st) {
+bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st) {
     ChanPlan &c = P->chan;
     if (!c.V || P->split_off) return false;  // (a slab's memory is budgeted without this scratch)
     if (!chan_alloc(&c.d_uc, c.uc_held, c.uc_bytes, st) || !chan_alloc(&c.d_gt, c.gt_held, c.gt_bytes, st)) return false;
-    return c.nsplit == 1 || chan_alloc(&P->d_ru_split, P->ru_split_bytes, c.gt_bytes * c.nsplit, st);
+    return nsplit == 1 || chan_alloc(&P->d_ru_split, P->ru_split_bytes, c.gt_bytes * nsplit, st);
 }
 
 template <typename S>
@@ -577,8 +657,8 @@ static dr_status pack(dr_plan *P, const void *u, int c0, int nc, cudaStream_t st
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "pack_kernel launch");
 }
 
-template <int V, int NW>
-static dr_status launch_t(dr_plan *P, float *ru, const RowMap &rows, size_t split_stride, int c0, int nc,
+template <int V, int NW, bool EO>
+static dr_status launch_t(dr_plan *P, float *ru, const RowMap &rows, size_t split_stride, int nsplit, int c0, int nc,
                           cudaStream_t st) {
     const ChanPlan &c = P->chan;
     constexpr int RW = chan_rw(V);
@@ -589,36 +669,45 @@ static dr_status launch_t(dr_plan *P, float *ru, const RowMap &rows, size_t spli
     if (!encode_tensor_map(&tr, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c.d_uc, dims, str, br) ||
         !encode_tensor_map(&tc, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c.d_uc, dims, str, bc))
         return fail(DR_ECUDA, "chan_fwd: tensor map encode failed");
-    auto kern = chan_fwd_kernel<V, RW, NW>;
+    auto kern = chan_fwd_kernel<V, RW, NW, EO>;
     const size_t smem = chan_ring(NW) + 128;
     const dr_status s = allow_dynamic_smem((const void *)kern, smem);
     if (s != DR_OK) return s;
     const ChanFwdArgs a{P->d_fold_fwd, c.d_blocks, ru, rows, split_stride, P->d_status, c.n, c.g, P->nx, P->ny,
                         P->ns, P->nz, c0, c.ms, c.spb, chan_ring(NW)};
-    const dim3 grid(c.nblocks * c.nbx, nc, c.nsplit);
+    const dim3 grid(c.nblocks * c.nbx, nc, nsplit);
     kern<<<grid, 32 * (NW + 1), smem, st>>>(tr, tc, a);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "chan_fwd_kernel launch");
 }
 
+template <bool EO>
+static dr_status launch_v(dr_plan *P, float *ru, size_t stride, int nsplit, int c0, int nc, cudaStream_t st) {
+    const ChanPlan &c = P->chan;
+    switch (c.V + (c.nw == 8 ? 0 : 8)) {
+        case 1: return launch_t<1, 8, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+        case 2: return launch_t<2, 8, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+        case 4: return launch_t<4, 8, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+        case 9: return launch_t<1, 16, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+        case 10: return launch_t<2, 16, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+        default: return launch_t<4, 16, EO>(P, ru, c.rows, stride, nsplit, c0, nc, st);
+    }
+}
+
 // Static transforms of all channels: into the channel-layout table, or the
 // split scratch when the march is cut into line chunks (the caller adds them).
-dr_status chan_static(dr_plan *P, const void *u, bool bf, cudaStream_t st, StaticOut &rs) {
+dr_status chan_static(dr_plan *P, const void *u, bool bf, bool eo, int nsplit, cudaStream_t st, StaticOut &rs) {
     ChanPlan &c = P->chan;
-    float *ru = (float *)(c.nsplit > 1 ? P->d_ru_split : c.d_gt);
+    float *ru = (float *)(nsplit > 1 ? P->d_ru_split : c.d_gt);
     const size_t stride = c.gt_bytes / sizeof(float);
     for (int c0 = 0; c0 < c.ncb; c0 += c.cb_pass) {
         const int nc = std::min(c.cb_pass, c.ncb - c0);
         dr_status s = bf ? pack<bf16>(P, u, c0, nc, st) : pack<float>(P, u, c0, nc, st);
         if (s != DR_OK) return s;
-        switch (c.V) {
-            case 1: s = c.nw == 8 ? launch_t<1, 8>(P, ru, c.rows, stride, c0, nc, st) : launch_t<1, 16>(P, ru, c.rows, stride, c0, nc, st); break;
-            case 2: s = c.nw == 8 ? launch_t<2, 8>(P, ru, c.rows, stride, c0, nc, st) : launch_t<2, 16>(P, ru, c.rows, stride, c0, nc, st); break;
-            default: s = c.nw == 8 ? launch_t<4, 8>(P, ru, c.rows, stride, c0, nc, st) : launch_t<4, 16>(P, ru, c.rows, stride, c0, nc, st); break;
-        }
+        s = eo ? launch_v<true>(P, ru, stride, nsplit, c0, nc, st) : launch_v<false>(P, ru, stride, nsplit, c0, nc, st);
         if (s != DR_OK) return s;
     }
-    rs = StaticOut{ru, c.rows, c.nsplit, stride};
+    rs = StaticOut{ru, c.rows, nsplit, stride};
     return DR_OK;
 }
 
@@ -631,11 +720,18 @@ void chan_free(dr_plan *P) {
 }  // namespace dr
 
 // For the parity tests (not part of the public header): run the automatic
-// forward of this plan on the channel kernel whatever the timing says.
-// Returns DR_EINVAL where the kernel does not take the plan.
-extern "C" dr_status dr_internal_use_channels(dr_plan *P) {
+// forward of this plan on the channel kernel whatever the timing says (the
+// operator calls and Chambolle-Pock; admm: ADMM's, in place of the fold in two
+// kernels).  Returns DR_EINVAL where the kernel does not take the plan.
+extern "C" dr_status dr_internal_use_channels(dr_plan *P, int admm) {
     if (!P || !P->chan.V) return dr::fail(DR_EINVAL, "no channel kernel for this plan");
-    P->chan.fwd = P->chan.fwd_st = 1;
+    if (admm) {
+        P->chan.eo = 1;
+        P->sel_fwd = 2;
+        P->sel_adj = 1;
+    } else {
+        P->chan.fwd = P->chan.fwd_st = 1;
+    }
     P->tuned = true;
     return DR_OK;
 }

@@ -1163,14 +1163,16 @@ dr_status fold_static_dispatch(dr_plan *P, const void *u, cudaStream_t st, Stati
     return fail(DR_EINVAL, "two-kernel folded forward: unsupported coefficient group");
 }
 
-// The forward in two steps: static transforms (chan: of the channel kernel),
-// then the distribution.
+// The forward in two steps: static transforms (chan: of the channel kernel,
+// 2 in the order of the thread-per-ray ones), then the distribution.
 template <typename S, typename T, int M>
 dr_status fold_fwd2_launch_t(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                             cudaStream_t st, bool chan) {
+                             cudaStream_t st, int chan) {
     StaticOut rs{};
     {
-        dr_status s = chan ? chan_static(P, u, sizeof(S) == 2, st, rs) : fold_static_dispatch<S, T, M>(P, u, st, rs);
+        dr_status s = chan ? chan_static(P, u, sizeof(S) == 2, chan == 2, chan == 2 ? fold2_chunks(P) : P->chan.nsplit,
+                                         st, rs)
+                           : fold_static_dispatch<S, T, M>(P, u, st, rs);
         if (s != DR_OK) return s;
     }
     fold_dist_kernel<S, T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
@@ -1246,7 +1248,7 @@ dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool 
 // ===========================================================================
 template <typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
-    fold_gram_kernel(const T *ru, T *gt, const T *__restrict__ gram, int nz, int U, int ns, int ms_ru, int m,
+    fold_gram_kernel(const T *ru, T *gt, const T *__restrict__ gram, int nz, int U, int ns, RowMap rin, int m,
                      int nsplit, size_t split_stride) {
     // ru and gt may be the same buffer (one chunk): each thread reads its row
     // whole before writing it, so they are not declared __restrict__
@@ -1254,8 +1256,10 @@ __global__ void __launch_bounds__(kRedThreads)
     constexpr bool V4 = sizeof(T) == 4;
     const size_t n = (size_t)nz * U * ns;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int a = (int)((i / ns) % U);
-        const T *r = ru + i * ms_ru;
+        const int z = (int)(i / ((size_t)U * ns));
+        const size_t ab = i - (size_t)z * U * ns;
+        const int a = (int)(ab / ns);
+        const T *r = ru + row_at(rin, z, ab);
         T rv[M];
         if constexpr (V4 && M % 4 == 0) {
             // rows are multiples of 4 floats from 16-byte aligned bases
@@ -1325,11 +1329,12 @@ __global__ void __launch_bounds__(kRedThreads)
 }
 
 template <typename S, typename T, int M>
-dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t st) {
+dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t st, bool chan) {
     if (!P->d_fold_gram) return fail(DR_EINVAL, "folded normal operator unavailable for this plan");
     StaticOut rs{};
     {
-        dr_status s = fold_static_dispatch<S, T, M>(P, x, st, rs);
+        dr_status s = chan ? chan_static(P, x, false, true, fold2_chunks(P), st, rs)
+                           : fold_static_dispatch<S, T, M>(P, x, st, rs);
         if (s != DR_OK) return s;
     }
     {
@@ -1337,7 +1342,7 @@ dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t 
         if (s != DR_OK) return s;
     }
     fold_gram_kernel<T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
-        (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows.ms, P->m,
+        (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows, P->m,
         rs.nsplit, rs.split_stride);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_gram_kernel launch");
@@ -1349,11 +1354,11 @@ struct FoldOps {
     static dr_status fwd(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                          cudaStream_t st);
     static dr_status fwd2(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                          cudaStream_t st, bool chan = false);
+                          cudaStream_t st, int chan = 0);
     static dr_status adj(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
                          cudaStream_t st);
     // y = R*R x on compute-typed buffers (static transforms, Gram mix, back-projection)
-    static dr_status normal(dr_plan *P, const void *x, void *y, cudaStream_t st);
+    static dr_status normal(dr_plan *P, const void *x, void *y, cudaStream_t st, bool chan = false);
 };
 
 #define DR_FOLD_DISPATCH(FN, S, T, ...)                   \
@@ -1377,7 +1382,7 @@ dr_status FoldOps<S, T>::fwd(dr_plan *P, const void *u, void *out, const void *g
 
 template <typename S, typename T>
 dr_status FoldOps<S, T>::fwd2(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                              cudaStream_t st, bool chan) {
+                              cudaStream_t st, int chan) {
     DR_FOLD_DISPATCH(fold_fwd2_launch_t, S, T, P, u, out, gm, mode, sigma, st, chan)
 }
 
@@ -1388,8 +1393,8 @@ dr_status FoldOps<S, T>::adj(dr_plan *P, const void *g, void *u, double alpha, d
 }
 
 template <typename S, typename T>
-dr_status FoldOps<S, T>::normal(dr_plan *P, const void *x, void *y, cudaStream_t st) {
-    DR_FOLD_DISPATCH(fold_normal_launch_t, S, T, P, x, y, st)
+dr_status FoldOps<S, T>::normal(dr_plan *P, const void *x, void *y, cudaStream_t st, bool chan) {
+    DR_FOLD_DISPATCH(fold_normal_launch_t, S, T, P, x, y, st, chan)
 }
 
 extern template struct FoldOps<float, float>;

@@ -50,11 +50,16 @@ dr_status launch_fwd_variant(dr_plan *P, int variant, bool calc, const void *u, 
         if (P->prec == DR_BF16_F32ACC && !calc) return FoldOps<bf16, float>::fwd(P, u, out, gm, mode, sigma, st);
         return FoldOps<float, float>::fwd(P, u, out, gm, mode, sigma, st);
     }
+    if (variant == kVarChanEO) {  // compute-typed (ADMM)
+        if (chan_fwd_ready(P, fold2_chunks(P), st))
+            return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st, 2);
+        variant = 2;  // no scratch to be had: the same values
+    }
     if (variant == kVarChan) {
-        if (chan_fwd_ready(P, st)) {
+        if (chan_fwd_ready(P, P->chan.nsplit, st)) {
             if (P->prec == DR_BF16_F32ACC && !calc)
-                return FoldOps<bf16, float>::fwd2(P, u, out, gm, mode, sigma, st, true);
-            return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st, true);
+                return FoldOps<bf16, float>::fwd2(P, u, out, gm, mode, sigma, st, 1);
+            return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st, 1);
         }
         // no scratch to be had (memory, a capture, a slab's budget)
         variant = calc || P->prec != DR_BF16_F32ACC ? P->sel_fwd : P->sel_fwd_st;
@@ -93,10 +98,13 @@ dr_status launch_adj_variant(dr_plan *P, int variant, bool calc, const void *g, 
 }
 
 // ADMM's forwards: its CG steps amplify the rounding of every sum, so the solver
-// keeps to the thread-per-ray kernels, whose sums it has always used, and its
-// iterates and objective stay what they are, bit for bit, whichever kernel is
-// the fastest one for a single call.
-static int fwd_choice(const dr_plan *P) { return P->var_fwd >= 0 ? P->var_fwd : P->sel_fwd; }
+// keeps the sums of the thread-per-ray kernels (by themselves, or the channel
+// kernel in their order), and its iterates and objective stay what they are, bit
+// for bit, whichever kernel is the fastest one for a single call.
+static int fwd_choice(const dr_plan *P) {
+    if (P->var_fwd >= 0) return P->var_fwd;
+    return P->sel_fwd == 2 && P->chan.eo ? kVarChanEO : P->sel_fwd;
+}
 // storage-typed calls on BF16 plans run the bf16-strip kernels, timed separately
 static int fwd_choice_st(const dr_plan *P) {
     if (P->var_fwd >= 0) return P->var_fwd;
@@ -138,9 +146,10 @@ dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, doub
 // static transforms are mixed per distinct angle and back-projected directly;
 // otherwise forward into gscratch, then adjoint.
 dr_status launch_normal_calc(dr_plan *P, const void *x, void *y, void *gscratch, cudaStream_t st) {
-    if (P->prec != DR_F64 && P->fold_U > 0 && P->fold2_ok && P->d_fold_gram && fwd_choice(P) == 2 &&
+    const int fc = fwd_choice(P);
+    if (P->prec != DR_F64 && P->fold_U > 0 && P->fold2_ok && P->d_fold_gram && (fc == 2 || fc == kVarChanEO) &&
         adj_choice(P) == 1)
-        return FoldOps<float, float>::normal(P, x, y, st);
+        return FoldOps<float, float>::normal(P, x, y, st, fc == kVarChanEO && chan_fwd_ready(P, fold2_chunks(P), st));
     dr_status s = launch_fwd_calc(P, x, gscratch, nullptr, 0, 0.0, st);
     if (s != DR_OK) return s;
     return launch_adj_calc(P, gscratch, y, 1.0, 0.0, st);
@@ -164,7 +173,7 @@ struct TuneKey {
 };
 struct TuneVal {
     int fwd, adj, lines, async, lines_st, async_st, f2_gi, f2_lines, f2_lines_st, fwd_st, f2_split, f2_async,
-        f2_async_st, adj_pp, f2_bv, f2_gi_st, chan_fwd, chan_fwd_st;
+        f2_async_st, adj_pp, f2_bv, f2_gi_st, chan_fwd, chan_fwd_st, chan_eo;
     double ms[5];
 };
 static std::mutex g_tune_mutex;
@@ -209,6 +218,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
             P->fold2_bv = it->second.f2_bv;
             P->chan.fwd = it->second.chan_fwd;
             P->chan.fwd_st = it->second.chan_fwd_st;
+            P->chan.eo = it->second.chan_eo;
             for (int i = 0; i < 5; ++i) P->tune_ms[i] = it->second.ms[i];
             P->tuned = true;
             return DR_OK;
@@ -620,11 +630,20 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->fold_adj_pp = best_pp;
     }
     // the channel kernel against the fastest of the others
-    P->chan.fwd = P->chan.fwd_st = 0;
-    if (chan_fwd_ready(P, st)) {
+    P->chan.fwd = P->chan.fwd_st = P->chan.eo = 0;
+    if (chan_fwd_ready(P, P->chan.nsplit, st)) {
         double t = 1e30;
         dr_status s = time_fwd(kVarChan, t);
         if (s != DR_OK) return s;
+        // ADMM's, with the line chunks just chosen: 8.5 against 16.3 ms for
+        // 8 x 1024^2, U = 300, m = 16; 0.54 against 0.50 ms for 16 x 256^2, U = 180,
+        // m = 8, whose CTAs leave the chip half empty without chunks
+        if (P->fold2_ok && chan_fwd_ready(P, fold2_chunks(P), st)) {
+            double te = 1e30;
+            s = time_fwd(kVarChanEO, te);
+            if (s != DR_OK) return s;
+            P->chan.eo = te < ms[4];
+        }
         P->chan.fwd = t < std::min(ms[0], std::min(ms[1], ms[4]));
         if (P->prec == DR_BF16_F32ACC) {  // (packs the stored values as floats)
             t = 1e30;
@@ -653,7 +672,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
                                                  P->fold_lines_st, P->fold_async_st, P->fold2_gi, P->fold2_lines,
                                                  P->fold2_lines_st, P->sel_fwd_st, P->fold2_split,
                                                  P->fold2_async, P->fold2_async_st, P->fold_adj_pp, P->fold2_bv,
-                                                 P->fold2_gi_st, P->chan.fwd, P->chan.fwd_st, {0, 0, 0, 0, 0}});
+                                                 P->fold2_gi_st, P->chan.fwd, P->chan.fwd_st, P->chan.eo, {0, 0, 0, 0, 0}});
     if (ins.second) {
         for (int i = 0; i < 5; ++i) ins.first->second.ms[i] = P->tune_ms[i];
     } else {  // another thread tuned the same problem first: follow its choice
@@ -675,6 +694,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->fold2_bv = ins.first->second.f2_bv;
         P->chan.fwd = ins.first->second.chan_fwd;
         P->chan.fwd_st = ins.first->second.chan_fwd_st;
+        P->chan.eo = ins.first->second.chan_eo;
     }
     return DR_OK;
 }

@@ -34,11 +34,11 @@ def _plan(case, prec, nt=3):
     return plan, oracle.Problem(nx, ny, nz, ns, theta, t, oracle.LEGENDRE, m, nt)
 
 
-def _force(plan):
+def _force(plan, admm=0):
     lib = dr.load()
-    lib.dr_internal_use_channels.argtypes = [ctypes.c_void_p]
+    lib.dr_internal_use_channels.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.dr_internal_use_channels.restype = ctypes.c_int
-    assert lib.dr_internal_use_channels(plan.handle) == dr.DR_OK
+    assert lib.dr_internal_use_channels(plan.handle, admm) == dr.DR_OK
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -82,6 +82,29 @@ def test_channel_forward_inside_solver():
     np.testing.assert_array_equal(us[0], us[1])
     uo, _ = P.chambolle_pock(g, np.zeros(us[0].shape), 5, 0.05, 1.0, L=L)
     assert rel(us[0], uo) <= 1e-5
+
+
+@pytest.mark.parametrize("case", CASES)
+@pytest.mark.parametrize("nsplit", [1, 3])
+def test_admm_on_channels_is_the_two_kernel_fold_bitwise(case, nsplit):
+    """In the order of the thread-per-ray kernels the channel kernel gives their
+    values bit for bit: residuals, CG products and the objective of a solve."""
+    if case[6] > 4 and min(case[:2]) < 8 * nsplit:
+        pytest.skip("fewer lines than chunks are worth")
+    g = dev_tensor(synth.random_g(synth.rng_for(4795), case[2], case[4], case[3]), dr.F32)
+    res = []
+    for channels in (True, False):
+        plan, _ = _plan(case, dr.F32)
+        plan.set_fold_march(nsplit)
+        if channels:
+            _force(plan, admm=1)
+        else:
+            plan.set_variant(dr.FOLD2, dr.FOLD)
+        u = torch.zeros(plan.u_shape(), dtype=torch.float32, device="cuda")
+        r = dr.admm_solve(plan, g, u, dr.solve_params(dr.ADMM_CG, iters=2, n_cg=2, lambda1=0.05, lambda2=1.0, rho=0.5))
+        res.append((host_values(u), r["objective"]))
+    np.testing.assert_array_equal(res[0][0], res[1][0])
+    np.testing.assert_array_equal(res[0][1], res[1][1])
 
 
 def test_captured_call_without_scratch():
