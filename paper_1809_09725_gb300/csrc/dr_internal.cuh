@@ -60,6 +60,7 @@ struct FwdProj {
 // coordinate of pixel (i, j) in bin-index units; cm = max(|c|, |s|).
 struct AdjProj {
     double c, s, C0, inv_c;
+    float cf, sf, e0, inv_c2;  // cos, sin, 1/cm - 1/(2 cm^2), 1/cm^2
 };
 
 // One distinct angle of the folded back-projection, with the float constants of

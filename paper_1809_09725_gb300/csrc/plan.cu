@@ -171,6 +171,10 @@ static AdjProj make_adj(double c, double s, double C0) {
     a.s = s;
     a.C0 = C0;
     a.inv_c = 1.0 / std::max(std::fabs(c), std::fabs(s));
+    a.cf = (float)c;
+    a.sf = (float)s;
+    a.e0 = (float)std::fma(-0.5 * a.inv_c, a.inv_c, a.inv_c);
+    a.inv_c2 = (float)(a.inv_c * a.inv_c);
     return a;
 }
 
@@ -402,8 +406,7 @@ static dr_status build_tables(dr_plan *P) {
             f.Af = (float)f.A; f.Bf = (float)f.B; f.Cf = (float)f.C; f.scale = (float)f.scale_d;
             ufw[a] = f;
             const AdjProj j = make_adj(c, s, -hx * c - hy * s + hs);
-            uad[a] = FoldAng{j.c, j.s, j.C0, (float)j.c, (float)j.s, (float)(16.0 * j.c),
-                             (float)std::fma(-0.5 * j.inv_c, j.inv_c, j.inv_c), (float)(j.inv_c * j.inv_c), 0.0f};
+            uad[a] = FoldAng{j.c, j.s, j.C0, j.cf, j.sf, 16.0f * j.cf, j.e0, j.inv_c2, 0.0f};
         }
         // forward work lists over unique angles
         const int M = P->M;

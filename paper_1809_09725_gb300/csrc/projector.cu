@@ -660,12 +660,12 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->sel_fwd = best;
         if (P->prec != DR_BF16_F32ACC) P->sel_fwd_st = best;
     }
-    // The folded back-projection has to win clearly: the two sum in different
-    // orders, which ADMM's CG steps amplify, so where they are close the solver
-    // keeps the direct one's sums.  Folded against direct, 16 x 256^2, K = 1800,
-    // m = 8: 0.36 : 1.61 ms for eight half-turns, 0.91 for three, 1.35 for two
-    // (on the line), 2.68 for one.
-    P->sel_adj = 1.2 * ms[3] < ms[2] ? 1 : 0;
+    // The folded back-projection has to win by a little: the two sum in different
+    // orders, which ADMM's CG steps amplify, so near a tie the choice should not
+    // follow the timer's noise.  Folded against direct, 16 x 256^2, K = 1800, m = 8:
+    // 0.36 : 1.44 ms for eight half-turns, 0.91 for three, 1.36 for two (on the
+    // line), 2.67 for one.
+    P->sel_adj = 1.05 * ms[3] < ms[2] ? 1 : 0;
     P->tuned = true;
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     auto ins = g_tune_cache.emplace(key, TuneVal{P->sel_fwd, P->sel_adj, P->fold_lines, P->fold_async,

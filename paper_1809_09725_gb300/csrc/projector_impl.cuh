@@ -17,8 +17,9 @@
 // per step, no float rounding of large coordinates, no float->int
 // conversion) and two scalar shared-memory taps per sample.
 //
-// Adjoint (adj_kernel): one CTA per (slice, 8*VPT x 16 voxel tile), 128
-// threads, VPT voxels per thread, all m accumulators per voxel in registers.
+// Adjoint (adj_kernel): one CTA per (ZS slices, 8*VPT x 16 voxel tile), 128
+// threads, VPT voxels of each slice per thread, all m accumulators per voxel in
+// registers.
 // Projections are consumed in stages of 32; for each stage one warp computes
 // where the tile's footprint falls on each detector row and issues one TMA
 // tile load per projection (a window of Wb bins, zero filled outside the
@@ -28,6 +29,7 @@
 // |sin|) and does m FMAs into the accumulators.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #pragma once
 #include "dr_device.cuh"
@@ -287,26 +289,46 @@ struct AdjShape {
 // Window geometry shared by host and device.
 __host__ __device__ inline int adj_align(int s_bytes) { return 16 / s_bytes; }
 
-template <typename S, typename T, int M>
-__global__ void __launch_bounds__(kAdjThreads)
+// Staging of the data windows: plain loads of all threads (bf16 rows of odd
+// length), TMA (rows of whole 16-byte vectors) or cp.async, element by element.
+enum AdjStaging { kAdjPlain, kAdjTma, kAdjCpAsync };
+
+// Issue bound: bins, fractions and weights take about 11 instructions per voxel
+// and projection, besides M multiply-adds.  ZS = 2 slices per thread share them,
+// and two coefficients share one multiply-add (fma.rn.f32x2, each half rounded by
+// itself).  Rows without 16-byte vectors are copied two stages ahead as well (they
+// were loaded between two barriers), and the float constants of an angle come
+// with the plan (a warp's FP64 instruction takes 59 clocks).  Every sum keeps its
+// terms and their order.
+//   4 x 256^2, K = 901, m = 32, rows of 257: 0.781 -> 0.617 ms
+//   16 x 256^2, K = 901, m = 16:             1.344 -> 1.108 ms
+//   6 x 128^2, K = 721, m = 8 (one slice):   0.154 -> 0.123 ms
+//   9 x 203 x 187, K = 721, m = 7, rows of 251: 0.314 -> 0.287 ms; two of three
+//   issue slots are used, by ten warps per SM (one slice per thread: 0.289 ms,
+//   twice the warps and 20 % more instructions)
+template <typename S, typename T, int M, int ZS>
+__global__ void __launch_bounds__(kAdjThreads, sizeof(T) == 8 ? 1 : (ZS == 2 ? 3 : 5))
     adj_kernel(const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_phi,
                const S *__restrict__ g, const T *__restrict__ phip, const AdjProj *__restrict__ proj,
-               S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int ns, int K, int m, int MP, int Wb,
-               int wbs, int use_tma, T alpha, T beta, int *status) {
+               S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int nz, int ns, int K, int m, int MP, int Wb,
+               int wbs, int staging, T alpha, T beta, int *status) {
     constexpr int VPT = AdjShape<M>::VPT;
     constexpr int TX = AdjShape<M>::TX;
     constexpr int TY = kAdjTY;
     constexpr int PP = kAdjP;
     constexpr int NST = kAdjStages;
     constexpr int ALIGN = 16 / (int)sizeof(S);
+    constexpr bool PK = sizeof(T) == 4 && M % 2 == 0;  // coefficient pairs
+    constexpr int NC = PK ? M / 2 : M;
+    using A = std::conditional_t<PK, unsigned long long, T>;
 
     extern __shared__ __align__(128) unsigned char adj_smem_raw[];
     // the launch adds 128 bytes so the base can be rounded up to 128 B (TMA destination alignment)
     // round up to 128 B by pointer arithmetic on the __shared__ array, so the
     // compiler keeps addressing it as shared memory (LDS, not generic loads)
     unsigned char *smem_raw = adj_smem_raw + ((128u - (smem_u32(adj_smem_raw) & 127u)) & 127u);
-    // per stage: window [PP][wbs] S (rows 128-B aligned), phi [PP][MP] T, prm [PP]
-    const size_t win_bytes = (size_t)PP * wbs * sizeof(S);
+    // per stage: window [ZS][PP][wbs] S (rows 128-B aligned), phi [PP][MP] T, prm [PP]
+    const size_t win_bytes = (size_t)ZS * PP * wbs * sizeof(S);
     const size_t phi_bytes = (((size_t)PP * MP * sizeof(T)) + 127) & ~(size_t)127;
     const size_t prm_bytes = (((size_t)PP * sizeof(AdjPrm<T>)) + 127) & ~(size_t)127;
     const size_t stage_bytes = win_bytes + phi_bytes + prm_bytes;
@@ -320,35 +342,36 @@ __global__ void __launch_bounds__(kAdjThreads)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ntx = (nx + TX - 1) / TX;
     const int x0 = (blockIdx.x % ntx) * TX, y0 = (blockIdx.x / ntx) * TY;
-    const int z = blockIdx.y;
+    const int z0 = blockIdx.y * ZS;
     const int xo = x0 + TX / 2, yo = y0 + TY / 2;  // tile origin voxel
     const int tx = tid & 7, ty = tid >> 3;
     const int dx0 = x0 + tx - xo, dy = y0 + ty - yo;
     const int nkb = (K + PP - 1) / PP;
 
     // Compute one projection's window and parameters (one lane per projection).
-    auto stage_params = [&](int st, int kb, int p, int &wb0_out, int &krow) {
+    auto stage_params = [&](int st, int kb, int p, int &wb0_out, int &kk_out) {
         const int k = kb * PP + p;
         const int kk = k < K ? k : K - 1;
         const AdjProj a = proj[kk];
         const double posO = xo * a.c + yo * a.s + a.C0;
-        const double dxa = (double)(-TX / 2), dxb = (double)(TX / 2 - 1);
-        const double dya = (double)(-TY / 2), dyb = (double)(TY / 2 - 1);
-        const double emin = posO + fmin(dxa * a.c, dxb * a.c) + fmin(dya * a.s, dyb * a.s);
-        int wb0 = (int)floor(emin) - 1;
+        int wb0;
+        if constexpr (sizeof(T) == 4)
+            wb0 = (int)floorf((float)posO + fminf((-TX / 2) * a.cf, (TX / 2 - 1) * a.cf) +
+                              fminf((-TY / 2) * a.sf, (TY / 2 - 1) * a.sf)) - 1;
+        else
+            wb0 = (int)floor(posO + fmin((-TX / 2) * a.c, (TX / 2 - 1) * a.c) +
+                             fmin((-TY / 2) * a.s, (TY / 2 - 1) * a.s)) - 1;
         wb0 = (wb0 >= 0) ? (wb0 / ALIGN) * ALIGN : -(((-wb0) + ALIGN - 1) / ALIGN) * ALIGN;
         const double rel = posO - wb0;
         const double ri = floor(rel);
         AdjPrm<T> pr;
         if constexpr (sizeof(T) == 4) {
-            const float inv_c = (float)a.inv_c;
-            pr.c = (float)a.c;
-            pr.s = (float)a.s;
-            pr.c8 = (float)(8.0 * a.c);
+            pr.c = a.cf;
+            pr.s = a.sf;
+            pr.c8 = 8.0f * a.cf;
             pr.qb = (float)(rel - ri) - 0.5f;
-            pr.inv_c2 = (float)(a.inv_c * a.inv_c);
-            pr.e0 = (float)(a.inv_c - 0.5 * a.inv_c * a.inv_c);
-            (void)inv_c;
+            pr.inv_c2 = a.inv_c2;
+            pr.e0 = a.e0;
             pr.idx_base = (int)ri - kMagicInt;
             pr.pad_ = 0;
         } else {
@@ -362,41 +385,68 @@ __global__ void __launch_bounds__(kAdjThreads)
         }
         prm_s(st)[p] = pr;
         wb0_out = wb0;
-        krow = z * K + kk;
+        kk_out = kk;
     };
 
     // TMA producer: warp 0 fills stage st with projection block kb.
     auto issue = [&](int st, int kb) {
-        int wb0 = 0, krow = 0;
-        if (lane < PP) stage_params(st, kb, lane, wb0, krow);
+        int wb0 = 0, kk = 0;
+        if (lane < PP) stage_params(st, kb, lane, wb0, kk);
         __syncwarp();
         if (lane == 0)
-            mbar_arrive_expect_tx(&full[st], (unsigned)(PP * Wb * sizeof(S) + PP * MP * sizeof(T)));
+            mbar_arrive_expect_tx(&full[st], (unsigned)(ZS * PP * Wb * sizeof(S) + PP * MP * sizeof(T)));
         __syncwarp();
-        if (lane < PP) tma_load_2d(win_s(st) + (size_t)lane * wbs, &tm_g, wb0, krow, &full[st]);
+        if (lane < PP)
+#pragma unroll
+            for (int i = 0; i < ZS; ++i)  // (a slice beyond the volume: the last one again, not stored)
+                tma_load_2d(win_s(st) + (size_t)(i * PP + lane) * wbs, &tm_g, wb0, min(z0 + i, nz - 1) * K + kk,
+                            &full[st]);
         if (lane == 0) tma_load_2d(phi_s(st), &tm_phi, 0, kb * PP, &full[st]);
         if (lane != 0) mbar_arrive(&full[st]);
     };
 
-    // Plain-load staging (unaligned rows): all threads, synchronous.
+    // cp.async producer: each warp the windows of a quarter of the projections.
+    auto issue_async = [&](int st, int kb) {
+        constexpr int PW = PP / (kAdjThreads / 32);
+        int wb0 = 0, kk = 0;
+        if (lane < PW) stage_params(st, kb, warp * PW + lane, wb0, kk);
+        for (int q = 0; q < PW; ++q) {
+            const int p = warp * PW + q, w = __shfl_sync(0xffffffffu, wb0, q), kq = __shfl_sync(0xffffffffu, kk, q);
+#pragma unroll
+            for (int i = 0; i < ZS; ++i) {
+                const S *row = g + ((size_t)min(z0 + i, nz - 1) * K + kq) * ns;
+                S *dst = win_s(st) + (size_t)(i * PP + p) * wbs;
+                for (int c = lane; c < Wb; c += 32) {
+                    const bool in = (unsigned)(w + c) < (unsigned)ns;
+                    if constexpr (sizeof(S) >= 4) cp_async_zfill<sizeof(S)>(dst + c, in ? row + w + c : row, in);
+                }
+            }
+        }
+        const int nv = PP * MP * (int)sizeof(T) / 16, left = (K - kb * PP) * MP * (int)sizeof(T) / 16;
+        const char *src = reinterpret_cast<const char *>(phip + (size_t)kb * PP * MP);
+        for (int i = tid; i < nv; i += kAdjThreads)
+            cp_async_zfill<16>(reinterpret_cast<char *>(phi_s(st)) + 16 * i, i < left ? src + 16 * i : src, i < left);
+    };
+
+    // Plain-load staging: all threads, synchronous.
     __shared__ int wb0_s[PP];
     auto fill_plain = [&](int kb) {
         if (warp == 0) {
-            int wb0 = 0, krow = 0;
+            int wb0 = 0, kk = 0;
             if (lane < PP) {
-                stage_params(0, kb, lane, wb0, krow);
+                stage_params(0, kb, lane, wb0, kk);
                 wb0_s[lane] = wb0;
             }
         }
         __syncthreads();
         S *win = win_s(0);
-        for (int i = tid; i < PP * Wb; i += kAdjThreads) {
-            const int p = i / Wb, c = i - p * Wb;
+        for (int i = tid; i < ZS * PP * Wb; i += kAdjThreads) {
+            const int zp = i / Wb, c = i - zp * Wb, p = ZS == 1 ? zp : zp % PP, zi = ZS == 1 ? 0 : zp / PP;
             const int k = kb * PP + p;
             const int b = wb0_s[p] + c;
             S v = S(0.0f);
-            if (k < K && b >= 0 && b < ns) v = g[((size_t)z * K + k) * ns + b];
-            win[(size_t)p * wbs + c] = v;
+            if (k < K && b >= 0 && b < ns) v = g[((size_t)min(z0 + zi, nz - 1) * K + k) * ns + b];
+            win[(size_t)zp * wbs + c] = v;
         }
         T *ph = phi_s(0);
         for (int i = tid; i < PP * MP; i += kAdjThreads) {
@@ -407,7 +457,7 @@ __global__ void __launch_bounds__(kAdjThreads)
         __syncthreads();
     };
 
-    if (use_tma) {
+    if (staging == kAdjTma) {
         if (tid == 0) {
             for (int s = 0; s < NST; ++s) mbar_init(&full[s], 32);
             fence_mbar_init();
@@ -415,20 +465,36 @@ __global__ void __launch_bounds__(kAdjThreads)
         __syncthreads();
         if (warp == 0)
             for (int s = 0; s < NST && s < nkb; ++s) issue(s, s);
+    } else if (staging == kAdjCpAsync) {
+        for (int s = 0; s < NST - 1; ++s) {
+            if (s < nkb) issue_async(s, s);
+            cp_async_commit();
+        }
     }
 
-    T acc[VPT][M];
+    A acc[ZS][VPT][NC];
 #pragma unroll
-    for (int v = 0; v < VPT; ++v)
+    for (int i = 0; i < ZS; ++i)
 #pragma unroll
-        for (int j = 0; j < M; ++j) acc[v][j] = T(0);
+        for (int v = 0; v < VPT; ++v)
+#pragma unroll
+            for (int j = 0; j < NC; ++j) acc[i][v][j] = 0;
 
     const T dxf = (T)dx0, dyf = (T)dy;
     for (int kb = 0; kb < nkb; ++kb) {
-        const int st = use_tma ? (kb % NST) : 0;
+        const int st = staging == kAdjPlain ? 0 : kb % NST;
         bool bad = false;
-        if (use_tma) bad = !mbar_wait_bounded(&full[st], (unsigned)((kb / NST) & 1), status, 2000000000ull);
-        else fill_plain(kb);
+        if (staging == kAdjTma) {
+            bad = !mbar_wait_bounded(&full[st], (unsigned)((kb / NST) & 1), status, 2000000000ull);
+        } else if (staging == kAdjCpAsync) {
+            // this stage has landed, and every thread is done with the one before it
+            cp_async_wait<NST - 2>();
+            __syncthreads();
+            if (kb + NST - 1 < nkb) issue_async((kb + NST - 1) % NST, kb + NST - 1);
+            cp_async_commit();
+        } else {
+            fill_plain(kb);
+        }
         if (!bad) {
             const S *win = win_s(st);
             const T *phs = phi_s(st);
@@ -436,35 +502,47 @@ __global__ void __launch_bounds__(kAdjThreads)
             const int np = min(PP, K - kb * PP);
             for (int p = 0; p < np; ++p) {
                 const AdjPrm<T> a = prm[p];
-                T ph[M];
-                if constexpr (sizeof(T) == 4 && (M % 4) == 0) {
+                A ph[NC];
+                if constexpr (PK && M % 4 == 0) {
                     // phi rows are MP = M rounded up to 4 floats, 16-byte aligned
 #pragma unroll
                     for (int c = 0; c < M / 4; ++c) {
-                        const float4 v4 = reinterpret_cast<const float4 *>(phs + p * MP)[c];
-                        ph[4 * c] = v4.x;
-                        ph[4 * c + 1] = v4.y;
-                        ph[4 * c + 2] = v4.z;
-                        ph[4 * c + 3] = v4.w;
+                        const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(phs + p * MP)[c];
+                        ph[2 * c] = v.x;
+                        ph[2 * c + 1] = v.y;
                     }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < M; ++j) ph[j] = phs[p * MP + j];
+                    for (int j = 0; j < NC; ++j) ph[j] = reinterpret_cast<const A *>(phs + p * MP)[j];
                 }
-                const S *w = win + (size_t)p * wbs;
+                const S *w = win + p * wbs;
                 if constexpr (sizeof(T) == 4) {
+                    // (the float's bits count bins: their magic goes into the address)
+                    const S *wz[ZS];
+#pragma unroll
+                    for (int i = 0; i < ZS; ++i) wz[i] = w + i * PP * wbs + a.idx_base;
                     float q = fmaf(dyf, a.s, fmaf(dxf, a.c, a.qb));
 #pragma unroll
                     for (int v = 0; v < VPT; ++v) {
                         const float t = q + kMagic;
                         const float fl = t - kMagic;
                         const float d = q - fl;
-                        const int idx = __float_as_int(t) + a.idx_base;
+                        const int idx = __float_as_int(t);
                         const float w0 = fmaxf(0.0f, fmaf(-d, a.inv_c2, a.e0));
                         const float w1 = fmaxf(0.0f, fmaf(d, a.inv_c2, a.e0));
-                        const float val = fmaf(w1, ldc<float>(w + idx + 1), w0 * ldc<float>(w + idx));
 #pragma unroll
-                        for (int j = 0; j < M; ++j) acc[v][j] = fmaf(ph[j], val, acc[v][j]);
+                        for (int i = 0; i < ZS; ++i) {
+                            const S *wi = wz[i] + idx;
+                            const float val = fmaf(w1, ldc<float>(wi + 1), w0 * ldc<float>(wi));
+                            if constexpr (PK) {
+                                const A vv = pack_f2(val, val);
+#pragma unroll
+                                for (int j = 0; j < NC; ++j) acc[i][v][j] = fma_f2(ph[j], vv, acc[i][v][j]);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < NC; ++j) acc[i][v][j] = fmaf(ph[j], val, acc[i][v][j]);
+                            }
+                        }
                         q += a.c8;
                     }
                 } else {
@@ -478,13 +556,13 @@ __global__ void __launch_bounds__(kAdjThreads)
                         const T w1 = fmax(T(0), a.inv_c - (T(1) - d0) * a.inv_c2);
                         const T val = w0 * ldc<T>(w + idx) + w1 * ldc<T>(w + idx + 1);
 #pragma unroll
-                        for (int j = 0; j < M; ++j) acc[v][j] += ph[j] * val;
+                        for (int j = 0; j < M; ++j) acc[0][v][j] += ph[j] * val;
                         q += a.c8;
                     }
                 }
             }
         }
-        if (use_tma) {
+        if (staging == kAdjTma) {
             if (__syncthreads_or(bad)) {
                 // give up: let loads already in flight land (bounded), then leave
                 if (tid == 0)
@@ -493,40 +571,51 @@ __global__ void __launch_bounds__(kAdjThreads)
                 return;
             }
             if (warp == 0 && kb + NST < nkb) issue(st, kb + NST);
-        } else {
+        } else if (staging == kAdjPlain) {
             __syncthreads();
         }
     }
 
     // ---- epilogue: u = alpha * acc + beta * u ----
 #pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-        const int x = x0 + tx + 8 * v, y = y0 + ty;
-        if (x >= nx || y >= ny) continue;
-        const size_t base = (((size_t)z * ny + y) * nx + x) * m;
-        if (u_c) {
+    for (int i = 0; i < ZS; ++i)
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            const int x = x0 + tx + 8 * v, y = y0 + ty, z = z0 + i;
+            if (x >= nx || y >= ny || z >= nz) continue;
+            const size_t base = (((size_t)z * ny + y) * nx + x) * m;
+            T sum[M];
+            if constexpr (PK) {
+#pragma unroll
+                for (int j = 0; j < NC; ++j) unpack_f2(acc[i][v][j], sum[2 * j], sum[2 * j + 1]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < M; ++j) sum[j] = acc[i][v][j];
+            }
 #pragma unroll
             for (int j = 0; j < M; ++j)
                 if (j < m) {
-                    T r = alpha * acc[v][j];
-                    if (beta != T(0)) r += beta * u_c[base + j];
-                    u_c[base + j] = r;
-                }
-        } else {
-#pragma unroll
-            for (int j = 0; j < M; ++j)
-                if (j < m) {
-                    T r = alpha * acc[v][j];
-                    if (beta != T(0)) r += beta * ldc<T>(u_s + base + j);
-                    stc<T>(u_s + base + j, r);
+                    T r = alpha * sum[j];
+                    if (u_c) {
+                        if (beta != T(0)) r += beta * u_c[base + j];
+                        u_c[base + j] = r;
+                    } else {
+                        if (beta != T(0)) r += beta * ldc<T>(u_s + base + j);
+                        stc<T>(u_s + base + j, r);
+                    }
                 }
         }
-    }
 }
 
-template <typename S, typename T, int M>
-inline dr_status adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
-                              cudaStream_t st) {
+// TMA needs 16-byte aligned rows and base addresses.
+template <typename S>
+inline bool adj_aligned(const dr_plan *P, const void *g) {
+    return ((size_t)P->ns * sizeof(S)) % 16 == 0 && ((uintptr_t)g % 16) == 0 && ((uintptr_t)P->d_PhiP % 16) == 0;
+}
+
+template <typename S, typename T, int M, int ZS>
+inline dr_status adj_launch_zs(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
+                               cudaStream_t st) {
     constexpr int TX = AdjShape<M>::TX;
     const int ALIGN = 16 / (int)sizeof(S);
     const double ext = std::sqrt((double)(TX - 1) * (TX - 1) + (double)(kAdjTY - 1) * (kAdjTY - 1));
@@ -534,17 +623,14 @@ inline dr_status adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, 
     Wb = (Wb + ALIGN - 1) / ALIGN * ALIGN;
     const int row_bytes = (int)((Wb * sizeof(S) + 127) / 128 * 128);
     const int wbs = row_bytes / (int)sizeof(S);
-    const size_t win_bytes = (size_t)kAdjP * wbs * sizeof(S);
+    const size_t win_bytes = (size_t)ZS * kAdjP * wbs * sizeof(S);
     const size_t phi_bytes = (((size_t)kAdjP * P->MP * sizeof(T)) + 127) & ~(size_t)127;
     const size_t prm_bytes = (((size_t)kAdjP * sizeof(AdjPrm<T>)) + 127) & ~(size_t)127;
     const size_t smem = (win_bytes + phi_bytes + prm_bytes) * kAdjStages + 128;
 
-    // TMA needs 16-byte aligned rows and base addresses.
-    const bool aligned = ((size_t)P->ns * sizeof(S)) % 16 == 0 && ((uintptr_t)g % 16) == 0 &&
-                         ((uintptr_t)P->d_PhiP % 16) == 0;
     CUtensorMap tm_g{}, tm_phi{};
-    int use_tma = 0;
-    if (aligned) {
+    int staging = sizeof(S) >= 4 ? kAdjCpAsync : kAdjPlain;
+    if (adj_aligned<S>(P, g)) {
         const CUtensorMapDataType dt = sizeof(S) == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
                                        : sizeof(S) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                                         : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -554,22 +640,38 @@ inline dr_status adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, 
                                               (uint64_t)P->nz * P->K, (uint64_t)P->ns * sizeof(S), (uint32_t)Wb, 1);
         const bool ok2 = encode_tensor_map_2d(&tm_phi, dtp, P->d_PhiP, (uint64_t)P->MP, (uint64_t)P->K,
                                               (uint64_t)P->MP * sizeof(T), (uint32_t)P->MP, (uint32_t)kAdjP);
-        use_tma = (ok1 && ok2) ? 1 : 0;
+        if (ok1 && ok2) staging = kAdjTma;
     }
-    auto kern = adj_kernel<S, T, M>;
+    auto kern = adj_kernel<S, T, M, ZS>;
     {
         dr_status s = allow_dynamic_smem((const void *)kern, smem);
         if (s != DR_OK) return s;
     }
     const int ntx = (P->nx + TX - 1) / TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
-    dim3 grid(ntx * nty, P->nz);
+    dim3 grid(ntx * nty, (P->nz + ZS - 1) / ZS);
     kern<<<grid, kAdjThreads, smem, st>>>(tm_g, tm_phi, (const S *)g, (const T *)P->d_PhiP, P->d_adj,
                                           u_calc ? nullptr : (S *)u, u_calc ? (T *)u : nullptr, P->nx, P->ny,
-                                          P->ns, P->K, P->m, P->MP, Wb, wbs, use_tma, (T)alpha, (T)beta,
+                                          P->nz, P->ns, P->K, P->m, P->MP, Wb, wbs, staging, (T)alpha, (T)beta,
                                           P->d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "adj_kernel launch");
     return DR_OK;
+}
+
+// Two slices per thread once that still leaves every SM two CTAs (4 x 300 x 256,
+// m = 4, 2.1 of them: 0.240 ms, one slice 0.258), unless the data has to be staged
+// by plain loads between barriers, which more CTAs hide (the volume above with
+// bf16 rows of 251: 0.329 ms against 0.406).
+template <typename S, typename T, int M>
+inline dr_status adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
+                              cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) {
+        constexpr int TX = AdjShape<M>::TX;
+        const long long tiles = (long long)((P->nx + TX - 1) / TX) * ((P->ny + kAdjTY - 1) / kAdjTY);
+        if (P->nz > 1 && tiles * ((P->nz + 1) / 2) >= 2 * P->num_sms && (sizeof(S) >= 4 || adj_aligned<S>(P, g)))
+            return adj_launch_zs<S, T, M, 2>(P, g, u, alpha, beta, u_calc, st);
+    }
+    return adj_launch_zs<S, T, M, 1>(P, g, u, alpha, beta, u_calc, st);
 }
 
 
