@@ -325,7 +325,8 @@ def launches_per_iteration(info, n_cg):
     both folded, a CG step's R*R p is the folded normal operator: static
     transforms, Gram mix, back-projection), n_cg + 1 D^T D (right-hand side +
     CG steps), prox, D^T w, n_cg updates, n_cg - 1 direction updates, the
-    fidelity dot and the iteration counter."""
+    fidelity dot and the iteration counter.  A lower bound where the channel-lane
+    forward runs: its packing of the volume is not counted."""
     adj_launches = 2 if info["adj_variant"] == 1 else 1
     fwd_launches = 2 if info["fwd_variant"] == 2 else 1
     normal_launches = 3 if (info["fwd_variant"], info["adj_variant"]) == (2, 1) else fwd_launches + adj_launches
