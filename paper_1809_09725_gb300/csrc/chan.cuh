@@ -30,11 +30,11 @@ struct StaticOut {
     size_t split_stride;
 };
 
-// forward variant of automatic operator calls and Chambolle-Pock, where the
-// autotuner found it faster (reported as the fold in two kernels)
+// forward variant of automatic operator calls, where the autotuner found it
+// faster (reported as the fold in two kernels)
 constexpr int kVarChan = 3;
 // the same kernel in the summation order, and with the line chunks, of the fold
-// in two kernels, whose values it then gives bit for bit (ADMM)
+// in two kernels, whose values it then gives bit for bit (the solvers)
 constexpr int kVarChanEO = 4;
 inline int fold2_chunks(const dr_plan *P) { return P->split_off ? 1 : (P->fold2_split > 1 ? P->fold2_split : 1); }
 constexpr int kChanWarps = 16;  // compute warps per CTA, at most (8: two CTAs per SM); one more copies

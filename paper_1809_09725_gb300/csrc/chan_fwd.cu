@@ -27,7 +27,7 @@
 // EO: the same march in the order of the thread-per-ray kernels (a sample's even
 // pixel is added before its odd one): the even and the odd pixel keep their own
 // registers, and the lanes work out weights and steps of a line's rays side by
-// side.  Bit for bit the fold in two kernels, so ADMM can run on it; 0.44 ms
+// side.  Bit for bit the fold in two kernels, so the solvers can run on it; 0.44 ms
 // (three line chunks) and 8.5 ms on the two volumes above.
 #include <algorithm>
 #include <cmath>
@@ -721,8 +721,7 @@ void chan_free(dr_plan *P) {
 
 // For the parity tests (not part of the public header): run the automatic
 // forward of this plan on the channel kernel whatever the timing says (the
-// operator calls and Chambolle-Pock; admm: ADMM's, in place of the fold in two
-// kernels).  Returns DR_EINVAL where the kernel does not take the plan.
+// operator calls; admm: the solvers', in place of the fold in two kernels).  Returns DR_EINVAL where the kernel does not take the plan.
 extern "C" dr_status dr_internal_use_channels(dr_plan *P, int admm) {
     if (!P || !P->chan.V) return dr::fail(DR_EINVAL, "no channel kernel for this plan");
     if (admm) {

@@ -170,7 +170,7 @@ struct ChanPlan {
     int V = 0, C = 0, ms = 0, spb = 0, ncb = 0;  // channels per lane / block, row length, slices per block, blocks
     int nw = 0, n = 0, g = 0, nblocks = 0, nbx = 0;  // warps, angles x runs of bins per CTA; angle blocks, bin blocks
     int nsplit = 1, cb_pass = 1;                 // line chunks; channel blocks packed at a time
-    int fwd = 0, fwd_st = 0, eo = 0;             // chosen by the autotuner (compute-typed / bf16-stored calls, ADMM)
+    int fwd = 0, fwd_st = 0, eo = 0;             // chosen by the autotuner (compute-typed / bf16-stored calls, the solvers)
     int *d_blocks = nullptr;
     RowMap rows{};
     size_t gt_bytes = 0, uc_bytes = 0;           // table of rows / packed volume

@@ -50,7 +50,7 @@ dr_status launch_fwd_variant(dr_plan *P, int variant, bool calc, const void *u, 
         if (P->prec == DR_BF16_F32ACC && !calc) return FoldOps<bf16, float>::fwd(P, u, out, gm, mode, sigma, st);
         return FoldOps<float, float>::fwd(P, u, out, gm, mode, sigma, st);
     }
-    if (variant == kVarChanEO) {  // compute-typed (ADMM)
+    if (variant == kVarChanEO) {  // compute-typed (the solvers)
         if (chan_fwd_ready(P, fold2_chunks(P), st))
             return FoldOps<float, float>::fwd2(P, u, out, gm, mode, sigma, st, 2);
         variant = 2;  // no scratch to be had: the same values
@@ -97,10 +97,12 @@ dr_status launch_adj_variant(dr_plan *P, int variant, bool calc, const void *g, 
     return fail(DR_EINVAL, "bad precision");
 }
 
-// ADMM's forwards: its CG steps amplify the rounding of every sum, so the solver
-// keeps the sums of the thread-per-ray kernels (by themselves, or the channel
-// kernel in their order), and its iterates and objective stay what they are, bit
-// for bit, whichever kernel is the fastest one for a single call.
+// The solvers' forwards: ADMM's CG steps amplify the rounding of every sum, and
+// the objective of either solver is a sum in double whose last digits a caller
+// reads.  So the solvers keep the sums of the thread-per-ray kernels (by
+// themselves, or the channel kernel in their order), and iterates and objective
+// stay what they are, bit for bit, in core and in slabs, whichever kernel is the
+// fastest one for a single call.
 static int fwd_choice(const dr_plan *P) {
     if (P->var_fwd >= 0) return P->var_fwd;
     return P->sel_fwd == 2 && P->chan.eo ? kVarChanEO : P->sel_fwd;
@@ -129,13 +131,6 @@ dr_status launch_adj(dr_plan *P, const void *g, void *u, double alpha, double be
 dr_status launch_fwd_calc(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                           cudaStream_t st) {
     return launch_fwd_variant(P, fwd_choice(P), true, u, out, gm, mode, sigma, st);
-}
-
-// Chambolle-Pock's forwards (no inner products: rounding is not amplified).
-dr_status launch_fwd_cp(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                        cudaStream_t st) {
-    const int v = P->var_fwd < 0 && P->chan.fwd ? kVarChan : fwd_choice(P);
-    return launch_fwd_variant(P, v, true, u, out, gm, mode, sigma, st);
 }
 
 dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, double beta, cudaStream_t st) {
@@ -635,7 +630,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         double t = 1e30;
         dr_status s = time_fwd(kVarChan, t);
         if (s != DR_OK) return s;
-        // ADMM's, with the line chunks just chosen: 8.5 against 16.3 ms for
+        // the solvers', with the line chunks just chosen: 8.5 against 16.3 ms for
         // 8 x 1024^2, U = 300, m = 16; 0.54 against 0.50 ms for 16 x 256^2, U = 180,
         // m = 8, whose CTAs leave the chip half empty without chunks
         if (P->fold2_ok && chan_fwd_ready(P, fold2_chunks(P), st)) {

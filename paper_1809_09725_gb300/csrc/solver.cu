@@ -353,8 +353,6 @@ dr_status launch_convert_bf16(dr_plan *P, const void *in, void *out, size_t n, b
 // The projector/TV launchers take "calc" (compute-typed) buffers here.
 dr_status launch_fwd_calc(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                           cudaStream_t st);
-dr_status launch_fwd_cp(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
-                        cudaStream_t st);
 dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, double beta, cudaStream_t st);
 
 // One ADMM-CG iteration (the captured sequence).
@@ -383,12 +381,12 @@ static dr_status cp_iteration(dr_plan *P, void *u, const void *g, const dr_solve
                               double tau, bool want_obj, cudaStream_t st) {
     Workspace &w = P->ws;
     const size_t ng = ng_elems(P);
-    TRY(launch_fwd_cp(P, w.ut, w.h1, g, 2, sigma, st));
+    TRY(launch_fwd_calc(P, w.ut, w.h1, g, 2, sigma, st));
     TRY(launch_cp_dual(P, w.ut, w.mu, sigma, prm.lambda1, prm.lambda2, st));
     TRY(launch_adj_calc(P, w.h1, w.q, 1.0, 0.0, st));
     TRY(launch_cp_primal(P, u, w.ut, w.q, w.mu, tau, prm.cp_theta, prm.lambda2, st));
     if (want_obj) {
-        TRY(launch_fwd_cp(P, u, w.gd, g, 1, 0.0, st));
+        TRY(launch_fwd_calc(P, u, w.gd, g, 1, 0.0, st));
         TRY(dot(P, w.gd, w.gd, ng, kSlotFid, w.obj, 1, 0, 0, st));
         TRY(launch_tv_sum(P, u, prm.lambda2, w.obj + 3, st));
     }
