@@ -781,7 +781,8 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjSh
 #pragma unroll
             for (int k = 0; k < TX / SX; ++k) {
                 const int xo = x0 + k * SX + SX / 2;
-                const double posO = xo * pj.c + yo * pj.s + pj.C0, fl = floor(posO);
+                // (written out, so that every tile shape rounds a subtile's middle alike)
+                const double posO = fma((double)xo, pj.c, yo * pj.s) + pj.C0, fl = floor(posO);
                 if (k == 0)  // the tile's lowest position, less a bin for rounding
                     wb0 = (int)fl - 1 + (int)floorf(fminf((-SX / 2) * pj.cf, (TX - 1 - SX / 2) * pj.cf) +
                                                     fminf((-TY / 2) * pj.sf, (TY / 2 - 1) * pj.sf));
