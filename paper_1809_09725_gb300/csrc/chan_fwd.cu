@@ -727,7 +727,7 @@ extern "C" dr_status dr_internal_use_channels(dr_plan *P, int admm) {
     if (admm) {
         P->chan.eo = 1;
         P->sel_fwd = 2;
-        P->sel_adj = 1;
+        P->sel_adj = P->solver_adj = 1;
     } else {
         P->chan.fwd = P->chan.fwd_st = 1;
     }

@@ -269,6 +269,7 @@ struct dr_plan {
     size_t gt_bytes = 0;
     int var_fwd = -1, var_adj = -1;   // -1 automatic, 0 direct, 1 fold, 2 fold in two kernels (forward)
     int sel_fwd = 0, sel_adj = 0;     // variant in use
+    int solver_adj = 0;               // the solvers' back-projection (a rule on the problem, not on times)
     bool tuned = false;
     double tune_ms[5] = {0, 0, 0, 0, 0}; // fwd direct, fwd fold, adj direct, adj fold, fwd fold (two kernels)
     double *d_partials = nullptr;
@@ -326,10 +327,10 @@ inline int red_grid(size_t n) {
 // out = (out + sigma R u - sigma gm) / (1 + sigma) (mode 2, CP dual h1).
 dr_status launch_fwd(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                      cudaStream_t st);
-// u = alpha R* g + beta u.  g and u are storage typed unless u_calc is set,
-// in which case u is a compute-typed (float/double) vector.
+// u = alpha R* g + beta u.  g and u are storage typed unless calc (g) or u_calc
+// (u) is set: compute-typed (float/double) vectors then.
 dr_status launch_adj(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
-                     cudaStream_t st);
+                     cudaStream_t st, bool calc = false);
 
 // TV family (tv.cu).  "calc" pointers are compute typed, storage pointers S.
 dr_status launch_grad(dr_plan *P, const void *u, bool u_calc, void *p, double lambda2, cudaStream_t st);

@@ -21,8 +21,6 @@
 
 namespace dr {
 
-dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, double beta, cudaStream_t st);
-
 // Filter.  A task is R rows by four consecutive outputs of each, in registers: a
 // step of four inputs takes four new taps (one vector, the lanes of a warp read
 // consecutive ones) and four inputs of each row (one broadcast vector a row) for
@@ -298,7 +296,7 @@ extern "C" dr_status dr_fbp_init(dr_plan *P, const void *g, void *u, int n_windo
     // back-project with Psi in place of Phi (kernels take the table pointer at launch)
     void *phi = P->d_PhiP;
     P->d_PhiP = P->d_fbp_phi;
-    if (P->prec == DR_BF16_F32ACC) s = launch_adj_calc(P, P->d_fbp_q, P->d_fbp_u, 1.0, 0.0, st);
+    if (P->prec == DR_BF16_F32ACC) s = launch_adj(P, P->d_fbp_q, P->d_fbp_u, 1.0, 0.0, true, st, true);
     else s = launch_adj(P, P->d_fbp_q, u, 1.0, 0.0, false, st);
     P->d_PhiP = phi;
     if (s != DR_OK) return s;

@@ -189,6 +189,34 @@ static dr_status upload(void **dst, const std::vector<double> &src, size_t &byte
     return DR_OK;
 }
 
+// Which back-projection the solvers run.  The folded and the direct one sum in
+// different orders, and a solve's objective (a sum in double) tells them apart
+// by a few 1e-7, so the choice must depend on the problem alone, not on a timer
+// near a tie nor on which kernel was made faster last: both kernels keep every
+// voxel's bits, this rule keeps a solve's.  The fold is taken while the distinct
+// angles (and kLaunch for its second launch) are at most the share of the
+// projections at which both took the same time.  Shares and the size where they
+// change are those of the kernels on which the results of solves were first
+// fixed; of 5373 shapes (48^2 to 700 x 512, 1 to 24 slices, m = 1 to 32, 180 to
+// 2880 projections, one to 30 projections per angle) 53 took the other kernel
+// there by more than 3 %, by a fifth at most.  The kernels of now (direct :
+// folded, 16 x 256^2, m = 8, K = 720): 0.600 : 0.564 ms for half as many angles,
+// where the rule stays direct, and 0.600 : 0.388 for a third.
+static bool solver_folds(const dr_plan *P, int U) {
+    constexpr int kSizes[8] = {1, 2, 4, 8, 12, 16, 24, 32};  // template sizes of m
+    // direct CTAs per SM up to which the first row of shares holds
+    constexpr double kFew[8] = {3.0, 2.1, 3.0, 3.0, 3.0, 4.9, 4.9, 2.7};
+    // rows of whole 16-byte vectors (the direct kernel brings them by TMA), others
+    constexpr double kShare[2][2][8] = {{{.60, .49, .51, .46, .44, .42, .43, .42}, {.60, .55, .535, .46, .44, .41, .37, .345}},
+                                        {{.80, .68, .66, .60, .54, .53, .60, .57}, {.80, .68, .66, .60, .54, .51, .45, .40}}};
+    constexpr int kLaunch = 6;
+    int i = 0;
+    while (i < 7 && kSizes[i] < P->M) ++i;
+    const int tx = P->M <= 8 ? 32 : (P->M <= 16 ? 16 : 8);
+    const double ctas = (double)((P->nx + tx - 1) / tx) * ((P->ny + kAdjTY - 1) / kAdjTY) * P->nz;
+    return U + kLaunch <= kShare[P->ns % 4 != 0][ctas > kFew[i] * P->num_sms][i] * P->K;
+}
+
 static dr_status build_tables(dr_plan *P) {
     const int K = P->K, m = P->m, MP = P->MP, MT = P->MT, nt = P->nt;
     const bool dbl = P->prec == DR_F64;
@@ -520,6 +548,7 @@ static dr_status build_tables(dr_plan *P) {
         P->sel_fwd = (P->fold_fwd_ok && fold < 0.8 * direct) ? 1 : 0;
         P->sel_fwd_st = P->sel_fwd;
         P->sel_adj = (fold < 0.8 * direct) ? 1 : 0;
+        P->solver_adj = solver_folds(P, U) ? 1 : 0;
     }
 
     // reductions, scalars, status

@@ -115,15 +115,16 @@ static int fwd_choice_st(const dr_plan *P) {
     return st ? P->sel_fwd_st : P->sel_fwd;
 }
 static int adj_choice(const dr_plan *P) { return P->var_adj >= 0 ? P->var_adj : P->sel_adj; }
+static int solver_adj_choice(const dr_plan *P) { return P->var_adj >= 0 ? P->var_adj : P->solver_adj; }
 
 dr_status launch_fwd(dr_plan *P, const void *u, void *out, const void *gm, int mode, double sigma,
                      cudaStream_t st) {
     return launch_fwd_variant(P, fwd_choice_st(P), false, u, out, gm, mode, sigma, st);
 }
 
-dr_status launch_adj(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
-                     cudaStream_t st) {
-    return launch_adj_variant(P, adj_choice(P), false, g, u, alpha, beta, u_calc, st);
+dr_status launch_adj(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc, cudaStream_t st,
+                     bool calc) {
+    return launch_adj_variant(P, adj_choice(P), calc, g, u, alpha, beta, u_calc, st);
 }
 
 // Compute-typed variants for the solvers: all buffers are float (F32 and
@@ -134,7 +135,7 @@ dr_status launch_fwd_calc(dr_plan *P, const void *u, void *out, const void *gm, 
 }
 
 dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, double beta, cudaStream_t st) {
-    return launch_adj_variant(P, adj_choice(P), true, g, u, alpha, beta, true, st);
+    return launch_adj_variant(P, solver_adj_choice(P), true, g, u, alpha, beta, true, st);
 }
 
 // y = R*R x: with the two-kernel folded forward and the folded adjoint, the
@@ -143,7 +144,7 @@ dr_status launch_adj_calc(dr_plan *P, const void *g, void *u, double alpha, doub
 dr_status launch_normal_calc(dr_plan *P, const void *x, void *y, void *gscratch, cudaStream_t st) {
     const int fc = fwd_choice(P);
     if (P->prec != DR_F64 && P->fold_U > 0 && P->fold2_ok && P->d_fold_gram && (fc == 2 || fc == kVarChanEO) &&
-        adj_choice(P) == 1)
+        solver_adj_choice(P) == 1)
         return FoldOps<float, float>::normal(P, x, y, st, fc == kVarChanEO && chan_fwd_ready(P, fold2_chunks(P), st));
     dr_status s = launch_fwd_calc(P, x, gscratch, nullptr, 0, 0.0, st);
     if (s != DR_OK) return s;
@@ -655,12 +656,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->sel_fwd = best;
         if (P->prec != DR_BF16_F32ACC) P->sel_fwd_st = best;
     }
-    // The folded back-projection has to win by a little: the two sum in different
-    // orders, which ADMM's CG steps amplify, so near a tie the choice should not
-    // follow the timer's noise.  Folded against direct, 16 x 256^2, K = 1800, m = 8:
-    // 0.36 : 1.44 ms for eight half-turns, 0.91 for three, 1.36 for two (on the
-    // line), 2.67 for one.
-    P->sel_adj = 1.05 * ms[3] < ms[2] ? 1 : 0;
+    P->sel_adj = ms[3] < ms[2] ? 1 : 0;
     P->tuned = true;
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     auto ins = g_tune_cache.emplace(key, TuneVal{P->sel_fwd, P->sel_adj, P->fold_lines, P->fold_async,
