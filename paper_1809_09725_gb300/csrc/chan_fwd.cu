@@ -328,9 +328,10 @@ __global__ void __launch_bounds__(32 * (NW + 1), NW == 8 ? 2 : 1)
             xl += bl;
             el += bl;
         }
-        if (!ok)  // a wait gave up: no copy of this CTA may outlive it
-            for (int i = oldest; i < k; ++i)
-                mbar_wait_bounded(&full[i % kChanSlots], (unsigned)((i / kChanSlots) & 1), P.status, 100000000ull);
+        // No copy of this CTA may outlive it: the compute warps leave as soon as any
+        // CTA's wait gave up, also after this warp has issued its last line.
+        for (int i = oldest; i < k; ++i)
+            mbar_wait_bounded(&full[i % kChanSlots], (unsigned)((i / kChanSlots) & 1), P.status, 100000000ull);
         return;
     }
 
