@@ -48,6 +48,7 @@ constexpr size_t kChanScratchMax = size_t(1) << 30;  // packed volume held at a 
 __host__ __device__ constexpr int chan_rw(int V) { return V == 4 ? 16 : 32; }
 __host__ __device__ constexpr int chan_boxes(int px) { return (px + kChanBox - 1) / kChanBox; }
 
+size_t split_bytes(const dr_plan *P);  // partial sums that the plan's choices need (projector.cu)
 dr_status chan_setup(dr_plan *P, const std::vector<FwdProj> &fw);
 bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st);
 // static transforms of u (bf: stored bf16, else float); chan_fwd_ready must hold

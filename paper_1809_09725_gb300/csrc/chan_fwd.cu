@@ -639,7 +639,11 @@ bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st) {
     ChanPlan &c = P->chan;
     if (!c.V || P->split_off) return false;  // (a slab's memory is budgeted without this scratch)
     if (!chan_alloc(&c.d_uc, c.uc_held, c.uc_bytes, st) || !chan_alloc(&c.d_gt, c.gt_held, c.gt_bytes, st)) return false;
-    return nsplit == 1 || chan_alloc(&P->d_ru_split, P->ru_split_bytes, c.gt_bytes * nsplit, st);
+    if (nsplit == 1) return true;
+    // (the buffer of partial sums is shared with the thread-per-ray kernels: never moved from here)
+    const size_t need = c.gt_bytes * nsplit;
+    if (P->d_ru_split) return P->ru_split_bytes >= need;
+    return chan_alloc(&P->d_ru_split, P->ru_split_bytes, std::max(need, split_bytes(P)), st);
 }
 
 template <typename S>

@@ -25,8 +25,25 @@ dr_status ensure_fold_scratch(dr_plan *P) {
     return DR_OK;
 }
 
+// What the plan's choices need for partial sums of a split march: chunks of the
+// thread-per-ray rows, or of the channel kernel's padded ones.
+size_t split_bytes(const dr_plan *P) {
+    const int n = P->fold2_ok ? fold2_chunks(P) : 1;
+    size_t b = 0;
+    if (n > 1) b = sizeof(float) * (size_t)P->nz * P->fold_U * P->ns * ((P->m + 3) / 4 * 4) * n;
+    if (P->chan.V && !P->split_off) {
+        if ((P->chan.fwd || P->chan.fwd_st) && P->chan.nsplit > 1) b = std::max(b, P->chan.gt_bytes * P->chan.nsplit);
+        if (P->chan.eo && n > 1) b = std::max(b, P->chan.gt_bytes * n);
+    }
+    return b;
+}
+
+// One buffer serves all of them, so its first allocation is for the largest: a
+// recorded graph may hold its address, and a later call of another kernel must
+// not move it.  (Only a new choice of chunks, or the autotuner, does.)
 dr_status ensure_split_scratch(dr_plan *P, size_t bytes) {
     if (P->d_ru_split && P->ru_split_bytes >= bytes) return DR_OK;
+    bytes = std::max(bytes, split_bytes(P));
     if (P->d_ru_split) {
         cudaError_t e = cudaFree(P->d_ru_split);
         P->d_ru_split = nullptr;
@@ -40,6 +57,16 @@ dr_status ensure_split_scratch(dr_plan *P, size_t bytes) {
     }
     P->ru_split_bytes = bytes;
     return DR_OK;
+}
+
+// Hold exactly what the choices need (trials of the autotuner grew it).
+static dr_status trim_split_scratch(dr_plan *P) {
+    const size_t keep = split_bytes(P);
+    if (!P->d_ru_split || P->ru_split_bytes == keep) return DR_OK;
+    cudaFree(P->d_ru_split);
+    P->d_ru_split = nullptr;
+    P->ru_split_bytes = 0;
+    return keep ? ensure_split_scratch(P, keep) : DR_OK;
 }
 
 // variant 0: direct (every projection at its own angle); 1: half-turn fold.
@@ -234,6 +261,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
     const size_t cs = calc_size(P->prec);
     DR_CUDA_TRY(cudaMemsetAsync(u_scratch, 0, nu_elems(P) * cs, st));
     DR_CUDA_TRY(cudaMemsetAsync(g_scratch, 0, ng_elems(P) * cs, st));
+    P->chan.fwd = P->chan.fwd_st = P->chan.eo = 0;
     double ms[5] = {1e30, 1e30, 1e30, 1e30, 1e30};
     double ms_st0 = 1e30, ms_st1 = 1e30, ms_st2 = 1e30;  // bf16-strip kernels of BF16 plans: direct, fold, fold in two
     // launches per trial: one warm-up, then the timed ones (reps - 1; the
@@ -511,17 +539,8 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
             }
             P->fold2_split = bs;
             P->fold2_bv = bbv;
-            // keep exactly the chosen chunks' scratch (the trials grew it to the largest)
-            const size_t keep = bs > 1 ? chunk * bs : 0;
-            if (P->d_ru_split && P->ru_split_bytes != keep) {
-                cudaFree(P->d_ru_split);
-                P->d_ru_split = nullptr;
-                P->ru_split_bytes = 0;
-                if (keep) {
-                    dr_status s = ensure_split_scratch(P, keep);
-                    if (s != DR_OK) return s;
-                }
-            }
+            dr_status s = trim_split_scratch(P);
+            if (s != DR_OK) return s;
         }
         // confirm the strip height against its neighbours with more timed
         // launches (neighbouring heights often differ by less than the noise
@@ -625,16 +644,24 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         }
         P->fold_adj_pp = best_pp;
     }
-    // the channel kernel against the fastest of the others
+    // the channel kernel against the fastest of the others (its trials may need
+    // more partial sums than were chosen above)
+    if (P->chan.V && P->d_ru_split) {
+        cudaFree(P->d_ru_split);
+        P->d_ru_split = nullptr;
+        P->ru_split_bytes = 0;
+    }
+    P->chan.fwd = P->chan.fwd_st = P->chan.eo = 1;  // (the scratch is sized for all of them)
+    const bool ready = chan_fwd_ready(P, P->chan.nsplit, st), ready_eo = P->fold2_ok && chan_fwd_ready(P, fold2_chunks(P), st);
     P->chan.fwd = P->chan.fwd_st = P->chan.eo = 0;
-    if (chan_fwd_ready(P, P->chan.nsplit, st)) {
+    if (ready) {
         double t = 1e30;
         dr_status s = time_fwd(kVarChan, t);
         if (s != DR_OK) return s;
         // the solvers', with the line chunks just chosen: 8.5 against 16.3 ms for
         // 8 x 1024^2, U = 300, m = 16; 0.54 against 0.50 ms for 16 x 256^2, U = 180,
         // m = 8, whose CTAs leave the chip half empty without chunks
-        if (P->fold2_ok && chan_fwd_ready(P, fold2_chunks(P), st)) {
+        if (ready_eo) {
             double te = 1e30;
             s = time_fwd(kVarChanEO, te);
             if (s != DR_OK) return s;
@@ -647,6 +674,10 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
             if (s != DR_OK) return s;
             P->chan.fwd_st = t < std::min(ms_st0, std::min(ms_st1, ms_st2));
         }
+    }
+    {
+        dr_status s = trim_split_scratch(P);
+        if (s != DR_OK) return s;
     }
     for (int i = 0; i < 5; ++i) P->tune_ms[i] = ms[i] < 1e29 ? ms[i] : -1.0;
     {

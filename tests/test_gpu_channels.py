@@ -127,3 +127,31 @@ def test_captured_call_without_scratch():
     dr.dyn_radon_fwd(plan, ud, g)
     plan.sync()
     assert_close(host_values(g), ref, 1e-5)
+
+
+def test_recorded_forward_outlives_a_solve():
+    """The partial sums of a forward recorded into a graph stay where they are when
+    a solve on the same plan needs more of them (padded rows in more chunks)."""
+    case = (128, 128, 5, 128, 360, 6, 8)
+    plan, P = _plan(case, dr.F32)
+    plan.set_fold_march(8)  # (the operator call's own chunks are four at most)
+    _force(plan, admm=1)
+    _force(plan)
+    u = synth.random_u(synth.rng_for(4797), case[2], case[1], case[0], case[6]).astype(np.float32)
+    ud = torch.from_numpy(u).cuda()
+    g, gr = (torch.zeros(plan.g_shape(), dtype=torch.float32, device="cuda") for _ in range(2))
+    dr.dyn_radon_fwd(plan, ud, g)
+    plan.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dr.dyn_radon_fwd(plan, ud, gr)
+    dr.dyn_radon_adj(plan, g, torch.empty(plan.u_shape(), dtype=torch.float32, device="cuda"))  # (its folded data)
+    held = plan.device_bytes()
+    x = torch.zeros(plan.u_shape(), dtype=torch.float32, device="cuda")
+    dr.admm_solve(plan, g, x, dr.solve_params(dr.ADMM_CG, iters=1, n_cg=1, lambda1=0.05, lambda2=1.0, rho=0.5))
+    assert plan.device_bytes() == held + plan.workspace_bytes(dr.ADMM_CG)
+    gr.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(host_values(gr), host_values(g))
+    assert_close(host_values(g), P.fwd(u.astype(np.float64)), 1e-5)
