@@ -597,10 +597,21 @@ __global__ void __launch_bounds__(kRedThreads)
 // Adjoint, step 1: fold the data per unique angle
 //   gt[z][a][b][j] = sum_{k in group(a)} phi_j(t_k) g[z][k][flip_k(b)]
 // ===========================================================================
+// wild[0] = 1 if a folded row holds an infinity or a NaN: the back-projection
+// then takes each voxel's bins by themselves (0 x infinity would spread).
+template <typename T, int N>
+__device__ __forceinline__ void note_wild(const T (&v)[N], int *wild) {
+    T f = T(0);
+#pragma unroll
+    for (int j = 0; j < N; ++j) f = fma(v[j], T(0), f);
+    if (f != T(0)) *(volatile int *)wild = 1;
+}
+
 template <typename S, typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
     fold_data_kernel(const S *__restrict__ g, T *__restrict__ gt, const int *__restrict__ start,
-                     const int *__restrict__ member, const T *__restrict__ phip, int nz, int U, int ns, int K, int MP) {
+                     const int *__restrict__ member, const T *__restrict__ phip, int nz, int U, int ns, int K, int MP,
+                     int *wild) {
     constexpr int MS = fold_ms(M);
     const size_t n = (size_t)nz * U * ns;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -645,6 +656,7 @@ __global__ void __launch_bounds__(kRedThreads)
                 }
             }
         }
+        note_wild(acc, wild);
         T *dst = gt + i * MS;
         if constexpr ((MS % 4) == 0 && sizeof(T) == 4) {
             float v[MS];
@@ -676,7 +688,9 @@ __global__ void __launch_bounds__(kRedThreads)
 // bin and angle by angle (ADMM amplifies any other rounding).  Angles whose sine
 // or cosine exceeds 0.99999, where the rounding of two positions could put
 // neighbouring taps two bins apart, read each voxel's two bins by themselves (a
-// CTA-uniform test per angle).
+// CTA-uniform test per angle), and so do all angles when the kernel that wrote
+// the folded data found an infinity or a NaN in it (status[1]; the last CTA to
+// finish, counted in status[2], clears it for the next call).
 // A quarter warp's lanes are 4 x 2 patches: their lowest bins span at most
 // 6 |cos| + 2 |sin| < 8 bins, and rows of an odd number of 16-byte slots then
 // never collide (lanes on the same bin share one broadcast).
@@ -685,14 +699,15 @@ __global__ void __launch_bounds__(kRedThreads)
 // (|position| <= 18 bins: the weights are exact to about 1e-6); a tile is one
 // or two of them.
 //
-// Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.293 ms;
-// 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.60 ms.  Shared memory, 90 % busy with
+// Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.296 ms;
+// 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.49 ms.  Shared memory, 90 % busy with
 // pairs, is at 65 %; what bounds it now is issue (56 % of the slots) together
 // with the skew of a CTA's warps at the stage barrier (24 % of the stalls; three
 // stages on mbarriers without it measured 0.300 and 6.62 ms).
 struct alignas(16) FoldPrm {
     float c, s, c16, e0;  // cos, sin, 16 cos, 1/cm - 1/(2 cm^2)  (cm = max(|c|, |s|))
-    float inv_c2, pad_[3];  // 1/cm^2
+    float inv_c2;           // 1/cm^2
+    float pad_[3];
     struct {
         float qb;  // fraction of a subtile's middle, less 1/2
         int idx;   // its bin in the window, less the float magic
@@ -723,6 +738,13 @@ struct FoldAdjShape {
 
 // Resident CTAs asked for: 4 ZS MC sums, 11 weight pairs and 4 bins per thread.
 __host__ __device__ constexpr int fold_adj_min_blocks(int sums) { return sums <= 4 ? 6 : (sums <= 8 ? 5 : 4); }
+
+// One thread of each CTA, when the CTA has read status[1] for the last time.
+__device__ __forceinline__ void fold_adj_done(int *status) {
+    __threadfence();
+    const unsigned last = gridDim.x * gridDim.y - 1;
+    if (atomicInc(reinterpret_cast<unsigned *>(status + 2), last) == last) *(volatile int *)(status + 1) = 0;
+}
 
 template <typename S, typename T, int M, int ZS>
 __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjShape<M>::MC))
@@ -804,6 +826,8 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjSh
         if (lane != 0) mbar_arrive(&full[st]);
     };
 
+    // |sin| or |cos| above which the voxels of a patch go by themselves
+    const float axis = __ldcg(status + 1) != 0 ? -1.0f : 0.99999f;
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) mbar_init(&full[s], 32);
         fence_mbar_init();
@@ -881,8 +905,8 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjSh
                 w1 = fmaxf(0.0f, fmaf(d, ic2, h.w));
                 return __float_as_int(t) + idx;
             };
-            if (fabsf(ac) > 0.99999f || fabsf(as) > 0.99999f) {
-                // close to an axis: each voxel's two bins by themselves
+            if (fabsf(ac) > axis || fabsf(as) > axis) {
+                // close to an axis, or bins that are not finite: each voxel's two bins by themselves
                 const float qv[4] = {qA, qB, qC, qD};
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
@@ -951,11 +975,13 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjSh
             if (tid == 0)
                 for (int s = kb; s < nkb && s < kb + NST; ++s)
                     mbar_wait_bounded(&full[s % NST], (unsigned)((s / NST) & 1), status, 100000000ull);
+            if (tid == 0) fold_adj_done(status);
             return;
         }
         // (the warps refill in turn: the others are already at the next stage)
         if (warp == (kb & 3) && kb + NST < nkb) issue(st, kb + NST);
     }
+    if (tid == 0) fold_adj_done(status);  // (behind the last stage's barrier)
     if (nk1 < nkb) flip();
 
 #pragma unroll
@@ -1197,7 +1223,7 @@ dr_status fold_adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, do
     // step 1: fold the data into the scratch buffer
     fold_data_kernel<S, T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const S *)g, (T *)gt, P->d_fold_start, P->d_fold_member, (const T *)P->d_PhiP, P->nz, P->fold_U, P->ns,
-        P->K, P->MP);
+        P->K, P->MP, P->d_status + 1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_data_kernel launch");
     return fold_backproject<S, T, M>(P, u, alpha, beta, u_calc, st, gt);
@@ -1250,7 +1276,7 @@ dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool 
 template <typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
     fold_gram_kernel(const T *ru, T *gt, const T *__restrict__ gram, int nz, int U, int ns, RowMap rin, int m,
-                     int nsplit, size_t split_stride) {
+                     int nsplit, size_t split_stride, int *wild) {
     // ru and gt may be the same buffer (one chunk): each thread reads its row
     // whole before writing it, so they are not declared __restrict__
     constexpr int MS = fold_ms(M);
@@ -1317,6 +1343,7 @@ __global__ void __launch_bounds__(kRedThreads)
             }
             ov[q] = acc;
         }
+        note_wild(ov, wild);
         T *dst = gt + i * MS;
         if constexpr (V4 && MS % 4 == 0) {
 #pragma unroll
@@ -1344,7 +1371,7 @@ dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t 
     }
     fold_gram_kernel<T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows, P->m,
-        rs.nsplit, rs.split_stride);
+        rs.nsplit, rs.split_stride, P->d_status + 1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_gram_kernel launch");
     return fold_backproject<S, T, M>(P, y, 1.0, 0.0, true, st);

@@ -555,12 +555,12 @@ static dr_status build_tables(dr_plan *P) {
     DR_CUDA_TRY(cudaMalloc(&P->d_partials, sizeof(double) * kRedSlots * kRedSlotStride));
     DR_CUDA_TRY(cudaMalloc(&P->d_counters, sizeof(unsigned) * kRedSlots));
     DR_CUDA_TRY(cudaMalloc(&P->d_scal, sizeof(DevScalars)));
-    DR_CUDA_TRY(cudaMalloc(&P->d_status, sizeof(int)));
+    DR_CUDA_TRY(cudaMalloc(&P->d_status, 3 * sizeof(int)));
     bytes += sizeof(double) * kRedSlots * kRedSlotStride + sizeof(unsigned) * kRedSlots + sizeof(DevScalars) +
-             sizeof(int);
+             3 * sizeof(int);
     DR_CUDA_TRY(cudaMemset(P->d_counters, 0, sizeof(unsigned) * kRedSlots));
     DR_CUDA_TRY(cudaMemset(P->d_scal, 0, sizeof(DevScalars)));
-    DR_CUDA_TRY(cudaMemset(P->d_status, 0, sizeof(int)));
+    DR_CUDA_TRY(cudaMemset(P->d_status, 0, 3 * sizeof(int)));
     return DR_OK;
 }
 
