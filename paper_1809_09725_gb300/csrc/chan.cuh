@@ -50,6 +50,7 @@ __host__ __device__ constexpr int chan_boxes(int px) { return (px + kChanBox - 1
 
 size_t split_bytes(const dr_plan *P);  // partial sums that the plan's choices need (projector.cu)
 dr_status chan_setup(dr_plan *P, const std::vector<FwdProj> &fw);
+bool chan_split_fits(const dr_plan *P, int nsplit);
 bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st);
 // static transforms of u (bf: stored bf16, else float); chan_fwd_ready must hold
 // (eo: each sample's even pixel first, the order of the thread-per-ray kernels)

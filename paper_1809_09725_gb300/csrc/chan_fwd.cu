@@ -589,10 +589,10 @@ dr_status chan_setup(dr_plan *P, const std::vector<FwdProj> &fw) {
     }
     // line chunks: fill the last wave, against the partial sums that every chunk
     // writes and the distribution adds
-    const size_t part = sizeof(float) * (size_t)c.ncb * c.C * U * P->ns;
+    c.gt_bytes = sizeof(float) * (size_t)c.ncb * c.C * U * P->ns;
     double best = 1e30;
     for (int s = 1; s <= 4; ++s) {
-        if (s > 1 && (part * s > split_budget(P->nz, P->K, P->ns, P->m) || std::min(P->nx, P->ny) < 16 * s)) break;
+        if (s > 1 && (!chan_split_fits(P, s) || std::min(P->nx, P->ny) < 16 * s)) break;
         const double ctas = (double)c.nblocks * c.nbx * c.ncb * s;
         const double cost = std::ceil(ctas / (P->num_sms * (c.nw == 8 ? 2 : 1))) / s * (1.0 + 0.04 * (s - 1));
         if (cost < best - 1e-9) {
@@ -601,7 +601,6 @@ dr_status chan_setup(dr_plan *P, const std::vector<FwdProj> &fw) {
         }
     }
     c.rows = RowMap{c.spb, c.C, c.ms, (size_t)U * P->ns * c.C};
-    c.gt_bytes = part;
     // The packed volume, as many blocks at a time as the scratch cap and the
     // memory a serving job is counted for leave (with few projections per
     // distinct angle there is none: the other kernels then)
@@ -635,9 +634,16 @@ static bool chan_alloc(void **p, size_t &held, size_t bytes, cudaStream_t st) {
     return true;
 }
 
+// Partial sums of nsplit line chunks within what a serving job is counted for (rows
+// padded to whole channel blocks are up to twice the thread-per-ray kernels').
+bool chan_split_fits(const dr_plan *P, int nsplit) {
+    return nsplit == 1 || P->chan.gt_bytes * nsplit <= split_budget(P->nz, P->K, P->ns, P->m);
+}
+
 bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st) {
     ChanPlan &c = P->chan;
     if (!c.V || P->split_off) return false;  // (a slab's memory is budgeted without this scratch)
+    if (!chan_split_fits(P, nsplit)) return false;
     if (!chan_alloc(&c.d_uc, c.uc_held, c.uc_bytes, st) || !chan_alloc(&c.d_gt, c.gt_held, c.gt_bytes, st)) return false;
     if (nsplit == 1) return true;
     // (the buffer of partial sums is shared with the thread-per-ray kernels: never moved from here)

@@ -33,7 +33,7 @@ size_t split_bytes(const dr_plan *P) {
     if (n > 1) b = sizeof(float) * (size_t)P->nz * P->fold_U * P->ns * ((P->m + 3) / 4 * 4) * n;
     if (P->chan.V && !P->split_off) {
         if ((P->chan.fwd || P->chan.fwd_st) && P->chan.nsplit > 1) b = std::max(b, P->chan.gt_bytes * P->chan.nsplit);
-        if (P->chan.eo && n > 1) b = std::max(b, P->chan.gt_bytes * n);
+        if (P->chan.eo && n > 1 && chan_split_fits(P, n)) b = std::max(b, P->chan.gt_bytes * n);
     }
     return b;
 }

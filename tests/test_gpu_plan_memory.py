@@ -43,3 +43,25 @@ def test_both_reports_of_device_memory_agree():
     _pair(plan)
     assert plan.device_bytes() > before
     assert plan.info()["device_bytes"] == plan.device_bytes()
+
+
+def test_solver_on_channels_stays_within_the_partial_sums_of_a_job():
+    """72 channels padded to 128: eight line chunks of them exceed what a job of this
+    size is counted for, so the solve stays on the fold in two kernels (same bits)
+    and holds what that holds."""
+    size = (32, 32, 9, 32, 150, 3, 8)
+    g = dev_tensor(synth.random_g(synth.rng_for(4971), 9, 150, 32), dr.F32)
+    held, us = [], []
+    for channels in (True, False):
+        plan = _plan(*size)
+        plan.set_fold_march(8)
+        if channels:
+            _use_channels(plan, 1)
+        else:
+            plan.set_variant(dr.FOLD2, dr.FOLD)
+        u = torch.zeros(plan.u_shape(), dtype=torch.float32, device="cuda")
+        dr.admm_solve(plan, g, u, dr.solve_params(dr.ADMM_CG, iters=2, n_cg=2, lambda1=0.05, lambda2=1.0, rho=0.5))
+        held.append(plan.device_bytes())
+        us.append(u.cpu().numpy())
+    assert held[0] == held[1]
+    np.testing.assert_array_equal(us[0], us[1])
