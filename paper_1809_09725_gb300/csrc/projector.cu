@@ -721,6 +721,15 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
     return DR_OK;
 }
 
+// The scratch of the channel kernels that were chosen, so that the calls to come
+// run on them from the first one on, recorded into a graph or not (without it
+// they run on the kernels of the thread-per-ray forms).
+static void hold_channel_scratch(dr_plan *P) {
+    const ChanPlan &c = P->chan;
+    if (c.fwd || c.fwd_st) chan_fwd_ready(P, c.nsplit, P->graph_stream);
+    if (c.eo) chan_fwd_ready(P, fold2_chunks(P), P->graph_stream);
+}
+
 }  // namespace dr
 
 using namespace dr;
@@ -772,6 +781,7 @@ dr_status dr_plan_autotune(dr_plan *P, double *times_ms) {
         cudaFree(gs);
         if (s != DR_OK) return s;
     }
+    hold_channel_scratch(P);
     if (times_ms)
         for (int i = 0; i < 5; ++i) times_ms[i] = P->tune_ms[i];
     return DR_OK;

@@ -65,3 +65,29 @@ def test_solver_on_channels_stays_within_the_partial_sums_of_a_job():
         us.append(u.cpu().numpy())
     assert held[0] == held[1]
     np.testing.assert_array_equal(us[0], us[1])
+
+
+@pytest.mark.parametrize("size", [(64, 64, 8, 64, 192, 8, 4), (128, 128, 6, 128, 720, 8, 8), (96, 80, 16, 101, 360, 6, 5),
+                                  (256, 256, 16, 256, 1800, 10, 8)])
+@pytest.mark.parametrize("prec", [dr.F32, dr.BF16])
+def test_first_forward_of_a_cached_plan_recorded_into_a_graph(size, prec):
+    """A plan that takes its choices from the cache has the scratch of the kernels
+    that won: its first forward, recorded into a graph, gives the bits of the plan
+    that timed them."""
+    timed = _plan(*size, prec)
+    timed.autotune()
+    cached = _plan(*size, prec)
+    cached.autotune()
+    dt = getattr(torch, timed.storage_dtype)
+    u = torch.randn(timed.u_shape(), device="cuda", generator=torch.Generator("cuda").manual_seed(3)).to(dt)
+    g, recorded = (torch.empty(timed.g_shape(), dtype=dt, device="cuda") for _ in range(2))
+    dr.dyn_radon_fwd(timed, u, g)
+    cached.set_variant(dr.FOLD2, dr.FOLD)  # (what the thread-per-ray forms allocate by themselves)
+    _pair(cached)
+    cached.set_variant(-1, -1)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dr.dyn_radon_fwd(cached, u, recorded)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(recorded, g)
