@@ -55,6 +55,7 @@ bool chan_fwd_ready(dr_plan *P, int nsplit, cudaStream_t st);
 // static transforms of u (bf: stored bf16, else float); chan_fwd_ready must hold
 // (eo: each sample's even pixel first, the order of the thread-per-ray kernels)
 dr_status chan_static(dr_plan *P, const void *u, bool bf, bool eo, int nsplit, cudaStream_t st, StaticOut &rs);
+void chan_release(dr_plan *P);
 void chan_free(dr_plan *P);
 
 inline RowMap slice_rows(size_t rows_per_slice, int ms) { return RowMap{1, ms, ms, rows_per_slice * ms}; }

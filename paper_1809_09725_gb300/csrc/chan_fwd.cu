@@ -722,6 +722,17 @@ dr_status chan_static(dr_plan *P, const void *u, bool bf, bool eo, int nsplit, c
     return DR_OK;
 }
 
+// Scratch of trials whose kernel was not chosen.
+void chan_release(dr_plan *P) {
+    ChanPlan &c = P->chan;
+    if (c.fwd || c.fwd_st || c.eo) return;
+    for (void **p : {&c.d_uc, &c.d_gt}) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+    c.uc_held = c.gt_held = 0;
+}
+
 void chan_free(dr_plan *P) {
     for (void *p : {(void *)P->chan.d_blocks, P->chan.d_uc, P->chan.d_gt})
         if (p) cudaFree(p);

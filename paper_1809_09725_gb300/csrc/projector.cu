@@ -676,6 +676,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         }
     }
     {
+        chan_release(P);
         dr_status s = trim_split_scratch(P);
         if (s != DR_OK) return s;
     }
@@ -717,6 +718,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         P->chan.fwd = ins.first->second.chan_fwd;
         P->chan.fwd_st = ins.first->second.chan_fwd_st;
         P->chan.eo = ins.first->second.chan_eo;
+        chan_release(P);
     }
     return DR_OK;
 }

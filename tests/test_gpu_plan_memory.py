@@ -91,3 +91,22 @@ def test_first_forward_of_a_cached_plan_recorded_into_a_graph(size, prec):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(recorded, g)
+
+
+@pytest.mark.parametrize("size", [(64, 64, 9, 64, 192, 8, 4), (128, 128, 7, 128, 720, 8, 8), (96, 80, 17, 101, 360, 6, 5),
+                                  (256, 256, 12, 256, 1800, 10, 8)])
+@pytest.mark.parametrize("prec", [dr.F32, dr.BF16])
+def test_timing_keeps_nothing_of_the_kernels_that_lost(size, prec):
+    """The plan that timed the kernels holds what a plan holds that takes the choices
+    from the cache, once both have run the forms that allocate on first use.
+    (Sizes that no other test has timed.)"""
+    held = []
+    for _ in range(2):
+        plan = _plan(*size, prec)
+        plan.autotune()
+        plan.set_variant(dr.FOLD2, dr.FOLD)
+        _pair(plan)
+        plan.set_variant(-1, -1)
+        _pair(plan)
+        held.append(plan.device_bytes())
+    assert held[0] == held[1]
