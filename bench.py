@@ -220,7 +220,10 @@ def algorithmic_smem_bytes(w, theta, variant, U):
     per voxel and distinct angle, two bins of the m folded sinograms from its
     staged window.  (The direct variants stage data per projection.)  The
     two-kernel folded forward (variant 2) reads the same samples in its
-    static-transform kernel."""
+    static-transform kernel.  With slices x coefficients on the lanes (variant
+    3) neighbouring rays share pixels: one new pixel vector per sample."""
+    if variant == 3:
+        return w.m * 4 * joseph_samples(theta, w.N, w.N, w.ns) * w.nz
     if variant in (1, 2):
         return 2 * w.m * 4 * joseph_samples(theta, w.N, w.N, w.ns) * w.nz
     return 2 * w.m * 4 * w.K * w.voxels()
@@ -236,8 +239,8 @@ def algorithmic_flops(w, variant, U):
     the interpolation for each of the m coefficients, plus m FMAs per
     detector sample to distribute (fold) over the K projections:
         2 (2 m U V + m K ns nz).
-    The two-kernel folded forward does the same arithmetic in two launches."""
-    if variant in (1, 2):
+    The two-kernel folded forwards do the same arithmetic in several launches."""
+    if variant in (1, 2, 3):
         return 2.0 * (2 * w.m * U * w.voxels() + w.m * w.K * w.ns * w.nz)
     return 2.0 * (w.m + 2) * w.K * w.voxels()
 
@@ -279,8 +282,9 @@ def roofline_of(w, theta, info, fwd_ms, adj_ms, tune=None):
     shared-memory bandwidth (side key)."""
     U = info["unique_angles"]
     if fwd_ms >= adj_ms:
-        variant = info["fwd_variant"]
-        kname = {1: "fold_fwd_kernel", 2: "fold_fwd_kernel(static)+fold_dist_kernel"}.get(variant, "fwd_kernel")
+        variant = info["fwd_variant_storage"]
+        kname = {1: "fold_fwd_kernel", 2: "fold_fwd_kernel(static)+fold_dist_kernel",
+                 3: "pack_kernel+chan_fwd_kernel+fold_dist_kernel"}.get(variant, "fwd_kernel")
         launch_ms = fwd_ms
         smem_bytes = algorithmic_smem_bytes(w, theta, variant, U)
     else:
@@ -295,12 +299,12 @@ def roofline_of(w, theta, info, fwd_ms, adj_ms, tune=None):
     hbm_peak, hbm_src = hbm_peak_gbs()
     hbm_gbs = hbm_bytes / (launch_ms * 1e-3) / 1e9
     smem_achieved = smem_bytes / (launch_ms * 1e-3) / 1e12
-    samples = joseph_samples(theta, w.N, w.N, w.ns) * w.nz if variant in (1, 2) else None
+    samples = joseph_samples(theta, w.N, w.N, w.ns) * w.nz if variant in (1, 2, 3) else None
     traffic = load_traffic(kname, w.name)
     return {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic,
             "algorithmic_flops_per_launch": flops,
-            "flops_formula": ("2 (2 m U V + m K ns nz), U distinct angles mod pi" if variant in (1, 2)
+            "flops_formula": ("2 (2 m U V + m K ns nz), U distinct angles mod pi" if variant in (1, 2, 3)
                               else "2 (m + 2) K V"),
             "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz (max SM clock)",
             "joseph_samples_per_launch": samples,
@@ -310,7 +314,7 @@ def roofline_of(w, theta, info, fwd_ms, adj_ms, tune=None):
                      "frac": smem_achieved / smem_peak_tbs(), "algorithmic_bytes": smem_bytes,
                      "peak_source": "derived: 152 SMs x 128 B/clk x 2.07 GHz"},
             "launch_ms": launch_ms, "fwd_ms": fwd_ms, "adj_ms": adj_ms,
-            "variants": {"unique_angles": U, "fwd": info["fwd_variant"], "adj": info["adj_variant"],
+            "variants": {"unique_angles": U, "fwd": info["fwd_variant_storage"], "adj": info["adj_variant"],
                          "fold2_group_threads_lines_split_async_rpt": [
                              info["fold2_group"], info["fold2_threads"], info["fold2_lines"],
                              info["fold2_split"], info["fold2_async"], info["fold2_rays_per_thread"]],
@@ -318,18 +322,21 @@ def roofline_of(w, theta, info, fwd_ms, adj_ms, tune=None):
                          "autotune_ms_fwd_direct_fold_adj_direct_fold_fwd_fold2": tune}}
 
 
-def launches_per_iteration(info, n_cg):
+def launches_per_iteration(variants, n_cg):
     """Kernels one ADMM-CG iteration launches: n_cg + 1 forwards and adjoints
     (the folded adjoint is two launches: data fold + back-projection; the
     two-kernel folded forward too: static transforms + distribution; with
     both folded, a CG step's R*R p is the folded normal operator: static
     transforms, Gram mix, back-projection), n_cg + 1 D^T D (right-hand side +
     CG steps), prox, D^T w, n_cg updates, n_cg - 1 direction updates, the
-    fidelity dot and the iteration counter.  A lower bound where the channel-lane
-    forward runs: its packing of the volume is not counted."""
-    adj_launches = 2 if info["adj_variant"] == 1 else 1
-    fwd_launches = 2 if info["fwd_variant"] == 2 else 1
-    normal_launches = 3 if (info["fwd_variant"], info["adj_variant"]) == (2, 1) else fwd_launches + adj_launches
+    fidelity dot and the iteration counter.  With slices x coefficients on the
+    lanes (forward variant 3) the volume is packed first, once per pass; one pass
+    is counted, a lower bound for volumes that take several.  `variants`: the
+    solvers' forward and adjoint."""
+    fwd, adj = variants
+    adj_launches = 2 if adj == 1 else 1
+    fwd_launches = {2: 2, 3: 3}.get(fwd, 1)
+    normal_launches = fwd_launches + (1 if fwd in (2, 3) and adj == 1 else adj_launches)
     per_iter = (1 + fwd_launches + adj_launches) + n_cg * (1 + normal_launches) + 2 * n_cg + 3
     return per_iter, fwd_launches
 
@@ -427,7 +434,7 @@ def run_ours(a):
     # the dominant kernels alone, on the same stream, in the variants the solver used
     fwd_ms, adj_ms = time_projectors(plan, dev, stream, reps=a.op_reps)
     roof = roofline_of(w, theta, info, fwd_ms, adj_ms, tune)
-    per_iter, fwd_launches = launches_per_iteration(info, w.n_cg)
+    per_iter, fwd_launches = launches_per_iteration(plan.solver_variants(), w.n_cg)
 
     # end to end through the public call with host buffers: each step is one
     # reconstruction job of e2e_iters iterations from pinned host memory

@@ -155,12 +155,17 @@ dr_status dr_plan_set_variant(dr_plan *plan, int fwd_variant, int adj_variant);
  * Time the variants of both projectors on this plan's geometry (allocates
  * and frees scratch; synchronises) and keep the fastest for automatic
  * selection; for the folded forwards also choose the strip height, staging
- * mode and coefficient group size (none changes the result).  The decision
- * is cached for the process, keyed by the sizes, basis, precision, angles and
- * times, so later plans of the same problem reuse it (same kernels,
- * bit-identical results) without timing again.  times_ms: HOST [5] nullable:
- * forward direct, forward fold, adjoint direct, adjoint fold, forward fold in
- * two kernels (-1 where a variant is unavailable).
+ * mode and coefficient group size (none changes the result).  The solvers take
+ * the forward's choice, in sums that do not depend on the kernel, and their
+ * adjoint by a rule (dr_plan_solver_variants).  The decision is cached for the
+ * process, keyed by the sizes, basis, precision, angles and times, so later
+ * plans of the same problem reuse it (same kernels, bit-identical results)
+ * without timing again; the call also allocates the scratch of the kernel with
+ * slices x coefficients on the lanes, if that was chosen (where there is no
+ * memory for it, dyn_radon_fwd runs the next fastest form, whose rounding
+ * differs).  times_ms: HOST [5] nullable: forward direct, forward fold, adjoint
+ * direct, adjoint fold, forward fold in two kernels (-1 where a variant is
+ * unavailable).
  */
 dr_status dr_plan_autotune(dr_plan *plan, double *times_ms);
 
@@ -234,8 +239,8 @@ dr_status dr_plan_set_fold_blocks(dr_plan *plan, int extra);
 typedef struct {
     int unique_angles;   /* distinct theta mod pi (0: the fold is unavailable) */
     int max_group;       /* most projections sharing one theta mod pi */
-    int fwd_variant;     /* variant the forward uses now (0 direct, 1 fold, 2 fold in two kernels) */
-    int adj_variant;     /* variant the adjoint uses now */
+    int fwd_variant;     /* variant of compute-typed forwards (0 direct, 1 fold, 2 fold in two kernels) */
+    int adj_variant;     /* variant dyn_radon_adj uses now */
     int tuned;           /* 1 once the variants have been timed */
     size_t device_bytes; /* device memory held by the plan */
     int fold_lines;      /* folded forward: image lines staged per shared-memory strip */
@@ -248,11 +253,23 @@ typedef struct {
     int fold2_async;     /* two-kernel folded forward: 1 if strips are double-buffered with cp.async */
     int fold_adj_angles; /* folded adjoint: distinct angles per pipeline stage */
     int fold2_angles;    /* two-kernel folded forward: distinct angles per CTA block */
-    int fwd_variant_storage; /* forward variant of storage-typed calls (differs on BF16 plans) */
+    int fwd_variant_storage; /* variant dyn_radon_fwd uses now: 0, 1, 2, or 3 = the fold in two kernels with
+                              * slices x coefficients on the lanes of a warp (automatic selection only) */
 } dr_plan_info_t;
 
 /* Describe the plan (host struct filled in). */
 dr_status dr_plan_info(const dr_plan *plan, dr_plan_info_t *info);
+
+/*
+ * The variants that the solvers run now (HOST ints).  They can differ from the
+ * operator calls' of dr_plan_info: CG steps amplify the rounding of every sum,
+ * so the solvers' sums must not depend on which kernel is the fastest one for a
+ * single call.  fwd: 0, 1, 2, or 3 where the kernel with slices x coefficients on
+ * the lanes gives variant 2's values bit for bit; adj: 0 or 1, by a rule on the
+ * plan's sizes and angles (the variant set with dr_plan_set_variant, if any).
+ * DR_EINVAL for NULL arguments.
+ */
+dr_status dr_plan_solver_variants(const dr_plan *plan, int *fwd, int *adj);
 
 /*
  * Wait for the plan's stream, then report any failure recorded by its
@@ -462,7 +479,8 @@ dr_status admm_solve_batch(int njobs, dr_plan *const *plans, const void *const *
  * streams.  The updated dual on the slice below a slab is carried over on the
  * device from the previous slab.  With the same operator norm (params->op_norm
  * > 0) the result is bit-identical to admm_solve with DR_CHAMBOLLE_POCK and
- * the same projector variants; otherwise the norm comes from a streamed power
+ * the same projector variants (dr_plan_solver_variants; 3 counts as 2, and the
+ * fold in two kernels marches in one line chunk here); otherwise the norm comes from a streamed power
  * iteration (params->power_iters passes over the volume), equal to the
  * in-core estimate up to rounding.
  *   plan     the whole volume's plan (nz = all slices); its stream is

@@ -30,8 +30,7 @@ struct StaticOut {
     size_t split_stride;
 };
 
-// forward variant of automatic operator calls, where the autotuner found it
-// faster (reported as the fold in two kernels)
+// forward variant of automatic operator calls, where the autotuner found it faster
 constexpr int kVarChan = 3;
 // the same kernel in the summation order, and with the line chunks, of the fold
 // in two kernels, whose values it then gives bit for bit (the solvers)

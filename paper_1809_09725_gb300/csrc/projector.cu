@@ -861,7 +861,7 @@ dr_status dr_plan_info(const dr_plan *P, dr_plan_info_t *info) {
     if (!P || !info) return fail(DR_EINVAL, "dr_plan_info: NULL argument");
     info->unique_angles = P->fold_U;
     info->max_group = P->fold_maxgrp;
-    info->fwd_variant = P->var_fwd >= 0 ? P->var_fwd : (P->chan.fwd ? 2 : P->sel_fwd);
+    info->fwd_variant = P->var_fwd >= 0 ? P->var_fwd : P->sel_fwd;
     info->adj_variant = P->var_adj >= 0 ? P->var_adj : P->sel_adj;
     info->tuned = P->tuned ? 1 : 0;
     info->device_bytes = dr_plan_device_bytes(P);
@@ -876,7 +876,15 @@ dr_status dr_plan_info(const dr_plan *P, dr_plan_info_t *info) {
     info->fold_adj_angles = P->fold_U > 0 ? P->fold_adj_pp : 0;
     info->fold2_angles =
         P->fold2_ok ? P->fold2_P[P->fold2_gi][P->d_fold2_blocks[P->fold2_gi][P->fold2_bv] ? P->fold2_bv : 0] : 0;
-    info->fwd_variant_storage = P->var_fwd >= 0 ? P->var_fwd : (P->chan.fwd_st ? 2 : P->sel_fwd_st);
+    info->fwd_variant_storage = fwd_choice_st(P) == kVarChan ? 3 : fwd_choice_st(P);
+    return DR_OK;
+}
+
+dr_status dr_plan_solver_variants(const dr_plan *P, int *fwd, int *adj) {
+    clear_error();
+    if (!P || !fwd || !adj) return fail(DR_EINVAL, "dr_plan_solver_variants: NULL argument");
+    *fwd = fwd_choice(P) == kVarChanEO ? 3 : fwd_choice(P);
+    *adj = solver_adj_choice(P);
     return DR_OK;
 }
 

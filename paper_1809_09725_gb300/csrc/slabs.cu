@@ -16,8 +16,9 @@
 //     of being re-read from the host (where the old value is already gone),
 //   * for the objective, the NEW u on slice z0-1 (carried the same way).
 // Every kernel computes each output element from the same inputs in the same
-// order as the whole-volume solver, so with the same operator norm the
-// result is the in-core Chambolle-Pock result bit for bit.
+// order as the whole-volume solver, so with the same operator norm and
+// projector variants (the fold in two kernels in one line chunk) the result is
+// the in-core Chambolle-Pock result bit for bit.
 //
 // Three device stages rotate: while slab q computes, slab q+1 is copied in
 // and slab q-1 is copied out, and the copy-in of q+1 need not wait for the

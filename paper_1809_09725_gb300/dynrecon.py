@@ -32,7 +32,7 @@ _STATUS = {DR_EINVAL: "EINVAL", DR_ENOMEM: "ENOMEM", DR_ECUDA: "ECUDA", DR_ETIME
 # Every symbol include/dynrecon.h declares.
 EXPORTS = ("dr_plan_create", "dr_plan_destroy", "dr_plan_set_stream", "dr_plan_device_bytes",
            "dr_plan_workspace_bytes", "dr_plan_state_bytes", "dr_plan_sync", "dr_plan_wait_selftest", "dr_plan_set_variant", "dr_plan_autotune",
-           "dr_plan_set_fold_strip", "dr_plan_set_fold_groups", "dr_plan_set_fold_march", "dr_plan_set_fold_adj_stage", "dr_plan_set_fold_blocks", "dr_plan_info",
+           "dr_plan_set_fold_strip", "dr_plan_set_fold_groups", "dr_plan_set_fold_march", "dr_plan_set_fold_adj_stage", "dr_plan_set_fold_blocks", "dr_plan_info", "dr_plan_solver_variants",
            "dyn_radon_fwd", "dyn_radon_adj", "dyn_radon_adj_noalloc", "dr_fbp_init", "tv4d_grad", "tv4d_grad_adj", "tv4d_normal",
            "tv4d_prox", "dr_solve_params_default", "admm_solve", "admm_solve_batch", "cp_solve_slabs",
            "cp_solve_slabs_device_bytes", "dr_job_device_bytes", "dr_job_slab_device_bytes", "dr_server_create",
@@ -122,6 +122,7 @@ def load(path: str = LIB_PATH):
         "dr_plan_set_fold_adj_stage": (i, [vp, i]),
         "dr_plan_set_fold_blocks": (i, [vp, i]),
         "dr_plan_info": (i, [vp, ctypes.POINTER(PlanInfo)]),
+        "dr_plan_solver_variants": (i, [vp, ctypes.POINTER(i), ctypes.POINTER(i)]),
         "dyn_radon_fwd": (i, [vp, vp, vp]),
         "dyn_radon_adj": (i, [vp, vp, vp, d]),
         "dyn_radon_adj_noalloc": (i, [vp, vp, vp, d]),
@@ -306,6 +307,12 @@ class Plan:
         inf = PlanInfo()
         _check(load().dr_plan_info(self._h, ctypes.byref(inf)))
         return {f: getattr(inf, f) for f, _ in PlanInfo._fields_}
+
+    def solver_variants(self):
+        """(forward, adjoint) variants of the solvers; forward 3: FOLD2's values by another kernel."""
+        fwd, adj = ctypes.c_int(), ctypes.c_int()
+        _check(load().dr_plan_solver_variants(self._h, ctypes.byref(fwd), ctypes.byref(adj)))
+        return fwd.value, adj.value
 
     def close(self):
         if self._h:

@@ -96,3 +96,19 @@ def test_solvers_back_projection_does_not_follow_the_timer(ht, adj, algo):
         res.append((host_values(u), r["objective"]))
     np.testing.assert_array_equal(res[0][0], res[1][0])
     np.testing.assert_array_equal(res[0][1], res[1][1])
+
+
+def test_plan_says_which_forward_runs():
+    """dyn_radon_fwd on the channel kernel is a variant of its own, and does not hide
+    what the solvers run."""
+    case = CASES[1]
+    plan = _plan(case)
+    own, solvers = plan.info()["fwd_variant"], plan.solver_variants()
+    assert solvers[0] == own
+    _use_channels(plan, 0)
+    assert plan.info()["fwd_variant_storage"] == 3
+    assert plan.info()["fwd_variant"] == own and plan.solver_variants() == solvers
+    _use_channels(plan, 1)
+    assert plan.info()["fwd_variant"] == dr.FOLD2 and plan.solver_variants() == (3, dr.FOLD)
+    plan.set_variant(dr.DIRECT, dr.DIRECT)
+    assert plan.info()["fwd_variant_storage"] == dr.DIRECT and plan.solver_variants() == (dr.DIRECT, dr.DIRECT)
