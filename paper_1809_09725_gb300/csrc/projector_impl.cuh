@@ -306,8 +306,17 @@ enum AdjStaging { kAdjPlain, kAdjTma, kAdjCpAsync };
 //   9 x 203 x 187, K = 721, m = 7, rows of 251: 0.314 -> 0.287 ms; two of three
 //   issue slots are used, by ten warps per SM (one slice per thread: 0.289 ms,
 //   twice the warps and 20 % more instructions)
+// CTAs per SM asked for.  One slice: as many as the registers of the sums allow (64
+// to 72 of them); with five, a grid of 1024 CTAs (4 x 256^2, m = 12) no longer fits
+// the chip at once, 0.281 against 0.247 ms.  FP64: four or five, as the one-slice
+// kernel takes without a bound; with one (163 registers at m = 32) 8 x 120^2,
+// K = 360, m = 32 took 4.71 ms, now 4.21.
+constexpr int adj_min_blocks(int bytes, int M, int ZS) {
+    return bytes == 8 ? (M == 4 || M == 8 || M == 16 ? 4 : 5) : (ZS == 2 ? 3 : (M == 12 || M == 24 ? 8 : 7));
+}
+
 template <typename S, typename T, int M, int ZS>
-__global__ void __launch_bounds__(kAdjThreads, sizeof(T) == 8 ? 1 : (ZS == 2 ? 3 : 5))
+__global__ void __launch_bounds__(kAdjThreads, adj_min_blocks(sizeof(T), M, ZS))
     adj_kernel(const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_phi,
                const S *__restrict__ g, const T *__restrict__ phip, const AdjProj *__restrict__ proj,
                S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int nz, int ns, int K, int m, int MP, int Wb,
@@ -658,17 +667,22 @@ inline dr_status adj_launch_zs(dr_plan *P, const void *g, void *u, double alpha,
     return DR_OK;
 }
 
-// Two slices per thread once that still leaves every SM two CTAs (4 x 300 x 256,
-// m = 4, 2.1 of them: 0.240 ms, one slice 0.258), unless the data has to be staged
-// by plain loads between barriers, which more CTAs hide (the volume above with
-// bf16 rows of 251: 0.329 ms against 0.406).
+// Two slices per thread once that leaves every SM two CTAs and does less work in
+// all: a CTA of two slices takes up to 1.8 times as long as one of one, so neither
+// an odd volume's empty slice nor a longer last round per SM may eat the gain
+// (m = 8, K = 360, one : two slices: 8 x 256^2 0.190 : 0.206 ms, 3 x 400^2
+// 0.190 : 0.222, 9 x 512^2 0.70 : 0.63).  Rows staged by plain loads between
+// barriers keep one slice: more CTAs hide them (9 x 203 x 187, m = 7, bf16 rows of
+// 251: 0.329 ms against 0.406).
 template <typename S, typename T, int M>
 inline dr_status adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, double beta, bool u_calc,
                               cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         constexpr int TX = AdjShape<M>::TX;
         const long long tiles = (long long)((P->nx + TX - 1) / TX) * ((P->ny + kAdjTY - 1) / kAdjTY);
-        if (P->nz > 1 && tiles * ((P->nz + 1) / 2) >= 2 * P->num_sms && (sizeof(S) >= 4 || adj_aligned<S>(P, g)))
+        const long long one = tiles * P->nz, two = tiles * ((P->nz + 1) / 2), sms = P->num_sms;
+        if (two >= 2 * sms && 18 * two < 10 * one && 18 * ((two + sms - 1) / sms) < 10 * ((one + sms - 1) / sms) &&
+            (sizeof(S) >= 4 || adj_aligned<S>(P, g)))
             return adj_launch_zs<S, T, M, 2>(P, g, u, alpha, beta, u_calc, st);
     }
     return adj_launch_zs<S, T, M, 1>(P, g, u, alpha, beta, u_calc, st);
