@@ -675,8 +675,10 @@ __global__ void __launch_bounds__(kRedThreads)
 // ===========================================================================
 // Adjoint, step 2: voxel-driven exact transpose of the folded sinograms
 // ===========================================================================
-// A thread holds a patch of 2 x 2 voxels for MC coefficients (all M up to 16;
-// half of them, and a second thread for the rest, above) of ZS slices.  The
+// A thread holds a patch of 2 x 2 voxels for MC coefficients (all M up to 16 and
+// half of them above, or half of that on small grids; other threads hold the rest)
+// of ZS slices (the weights, about as many instructions as 8 coefficients' sums,
+// serve all of them).  The
 // patch projects |cos| + |sin| <= sqrt 2 bins wide, so its eight taps lie in
 // four consecutive bins b .. b + 3 counted from the voxel that projects lowest:
 // that voxel takes bins 0 and 1, the two beside it two of bins 0 to 2, the one
@@ -714,30 +716,37 @@ struct alignas(16) FoldPrm {
     } sub[2];
 };
 
+//
+// NG threads share a patch's coefficients (a warp or more apart): one or two, or
+// twice as many where that many CTAs would leave the chip to a few long ones.
 template <int M>
+constexpr int kFoldAdjNG = M <= 16 ? 1 : 2;
+template <int M, int NG_>
 struct FoldAdjShape {
-    static constexpr int NG = M <= 16 ? 1 : 2;  // threads sharing a patch's coefficients
+    static constexpr int NG = NG_;
     static constexpr int MC = M / NG;
-    static constexpr int TX = NG == 1 ? 32 : 16;  // tile: TX x 16 voxels per CTA of 128 threads
+    static constexpr int TX = 32 / NG;  // tile: TX x 16 voxels per CTA of 128 threads
     static constexpr int SX = M <= 8 ? 32 : (M <= 16 ? 16 : 8);  // subtile
     // a row's position from the row above it (else from the subtile's middle)
     static constexpr bool STEP = M <= 16;
-    // bins of a window: the tile's extent at any angle (35 or 22), the patch's
+    // bins of a window: the tile's extent at any angle (35, 22 or 17), the patch's
     // fourth bin and a margin for the rounding of the first
-    static constexpr int WB = NG == 1 ? 41 : 28;
+    static constexpr int WB = NG == 1 ? 41 : (NG == 2 ? 28 : 24);
     // A window is one run of WB bins x MS floats of a sinogram row, copied in
     // boxes of at most 256 floats and whole 128-byte lines, one box row each (a
     // box of WB rows of MS floats fetched 2.7 times the bytes from L2).
     static constexpr int NBOX = (WB * fold_ms(M) + 255) / 256;
     static constexpr int BOX = ((WB * fold_ms(M) + NBOX - 1) / NBOX + 31) / 32 * 32;
     static constexpr int WIN = NBOX * BOX;  // floats
-    // slices a thread may take (the weights, about as many instructions as 8
-    // coefficients' sums, serve all of them)
-    static constexpr int ZS = M <= 4 ? 4 : (M <= 8 ? 2 : 1);
 };
 
 // Resident CTAs asked for: 4 ZS MC sums, 11 weight pairs and 4 bins per thread.
-__host__ __device__ constexpr int fold_adj_min_blocks(int sums) { return sums <= 4 ? 6 : (sums <= 8 ? 5 : 4); }
+// (With five for m = 5 to 8 smaller grids are 4 to 6 % faster, but 761 to 912 CTAs
+// take a second round: 7 x 256^2, m = 8, U = 120 0.126 ms, with six 0.119.)
+__host__ __device__ constexpr int fold_adj_min_blocks(int M, int NG, int ZS) {
+    const int sums = ZS * M / NG;
+    return sums <= 4 ? 7 : (sums <= 8 ? (M <= 8 ? 6 : 5) : 4);
+}
 
 // One thread of each CTA, when the CTA has read status[1] for the last time.
 __device__ __forceinline__ void fold_adj_done(int *status) {
@@ -746,12 +755,12 @@ __device__ __forceinline__ void fold_adj_done(int *status) {
     if (atomicInc(reinterpret_cast<unsigned *>(status + 2), last) == last) *(volatile int *)(status + 1) = 0;
 }
 
-template <typename S, typename T, int M, int ZS>
-__global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjShape<M>::MC))
+template <typename S, typename T, int M, int NG_, int ZS>
+__global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M, NG_, ZS))
     fold_adj_kernel(const __grid_constant__ CUtensorMap tm_gt, const FoldAng *__restrict__ ang,
                     S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int nz, int U, int U1, int m, T alpha,
                     T beta, int *status, int PP, int vec) {
-    using Sh = FoldAdjShape<M>;
+    using Sh = FoldAdjShape<M, NG_>;
     constexpr int TX = Sh::TX, TY = kAdjTY, SX = Sh::SX, NG = Sh::NG, MC = Sh::MC;
     constexpr int NST = kFoldAdjStages;
     constexpr int MS = fold_ms(M);
@@ -777,10 +786,11 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(ZS *FoldAdjSh
     const int ntx = (nx + TX - 1) / TX;
     const int x0 = (blockIdx.x % ntx) * TX, y0 = (blockIdx.x / ntx) * TY;
     const int z0 = blockIdx.y * ZS;
-    // patch of this thread: a warp covers 8 x 4 patches, a quarter of it 4 x 2
-    const int vw = NG == 1 ? warp : (warp & 1), cg = NG == 1 ? 0 : (warp >> 1);
-    const int px = (lane & 3) + 4 * ((lane >> 3) & 1) + (NG == 1 ? 8 * (vw & 1) : 0);
-    const int py = ((lane >> 2) & 1) + 2 * (lane >> 4) + 4 * (NG == 1 ? vw >> 1 : vw);
+    // patch of this thread: a warp covers 8 x 4 patches (tiles of 8 columns: 4 x 8),
+    // a quarter of it 4 x 2
+    const int vw = warp % (4 / NG), cg = warp / (4 / NG);
+    const int px = NG == 4 ? (lane & 3) : (lane & 3) + 4 * ((lane >> 3) & 1) + (NG == 1 ? 8 * (vw & 1) : 0);
+    const int py = NG == 4 ? lane >> 2 : ((lane >> 2) & 1) + 2 * (lane >> 4) + 4 * (NG == 1 ? vw >> 1 : vw);
     const int dx = 2 * px, dy = 2 * py;
     // blocks of PP angles: those with cos >= 0 (the first U1), then the others
     const int nk1 = (U1 + PP - 1) / PP, nkb = nk1 + (U - U1 + PP - 1) / PP;
@@ -1231,37 +1241,65 @@ dr_status fold_adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, do
 
 // Back-project the folded sinograms (step 2 of the folded adjoint):
 // u = alpha R*(folded) + beta u.
-template <typename S, typename T, int M>
-dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool u_calc, cudaStream_t st, void *gt) {
+template <typename S, typename T, int M, int NG, int ZS>
+dr_status fold_backproject_t(dr_plan *P, void *u, double alpha, double beta, bool u_calc, cudaStream_t st, void *gt) {
+    using Sh = FoldAdjShape<M, NG>;
     constexpr int MS = fold_ms(M);
-    if (!gt) gt = P->d_gt;
     CUtensorMap tm{};
     if (!encode_tensor_map_2d(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, gt, (uint64_t)P->ns * MS, (uint64_t)P->nz * P->fold_U,
-                              (uint64_t)P->ns * MS * sizeof(T), (uint32_t)FoldAdjShape<M>::BOX, 1))
+                              (uint64_t)P->ns * MS * sizeof(T), (uint32_t)Sh::BOX, 1))
         return fail(DR_ECUDA, "fold adj: tensor map encode failed");
-    constexpr int TX = FoldAdjShape<M>::TX, ZMAX = FoldAdjShape<M>::ZS;
-    const int ntx = (P->nx + TX - 1) / TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
-    // several slices per thread where that leaves every SM its resident CTAs
-    const int zs = ZMAX > 1 && (long long)ntx * nty * ((P->nz + ZMAX - 1) / ZMAX) >=
-                                   (long long)P->num_sms * fold_adj_min_blocks(ZMAX * FoldAdjShape<M>::MC)
-                       ? ZMAX : 1;
     // angles per pipeline stage: fewer shrink the windows' shared memory so that
     // more CTAs fit on an SM (the angles are summed in the same order)
-    constexpr int row_bytes = FoldAdjShape<M>::WIN * (int)sizeof(T);
-    const int pp = std::max(1, std::min(std::min(32, P->fold_adj_pp), kFoldAdjWin / (zs * row_bytes)));
-    const size_t stage = (size_t)pp * zs * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128);
+    constexpr int row_bytes = Sh::WIN * (int)sizeof(T);
+    const int pp = std::max(1, std::min(std::min(32, P->fold_adj_pp), kFoldAdjWin / (ZS * row_bytes)));
+    const size_t stage = (size_t)pp * ZS * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128);
     const size_t smem = stage * kFoldAdjStages + 128;
-    auto kern = zs > 1 ? fold_adj_kernel<S, T, M, ZMAX> : fold_adj_kernel<S, T, M, 1>;
+    auto kern = fold_adj_kernel<S, T, M, NG, ZS>;
     {
         dr_status s = allow_dynamic_smem((const void *)kern, smem);
         if (s != DR_OK) return s;
     }
-    dim3 grid(ntx * nty, (P->nz + zs - 1) / zs);
+    const int ntx = (P->nx + Sh::TX - 1) / Sh::TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
+    dim3 grid(ntx * nty, (P->nz + ZS - 1) / ZS);
     kern<<<grid, kAdjThreads, smem, st>>>(tm, P->d_fold_ang, u_calc ? nullptr : (S *)u, u_calc ? (T *)u : nullptr,
                                           P->nx, P->ny, P->nz, P->fold_U, P->fold_U1, P->m, (T)alpha, (T)beta, P->d_status, pp,
                                           P->m == M && ((uintptr_t)u & 15u) == 0);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "fold_adj_kernel launch");
+}
+
+// Which form, by the CTAs it makes (bits do not depend on it).
+//   m <= 8: several slices per thread once that leaves every SM two CTAs and is less
+//     work in all: a CTA of four slices (m <= 4) takes up to 2.3 times as long as one
+//     of one, of two up to 1.7, so neither a volume's last, partly empty group nor a
+//     longer last round per SM may eat the gain.  U = 120, one : several slices:
+//     m = 4: 4 x 512^2 0.160 : 0.126 ms, 2 x 700 x 512 0.118 : 0.172; m = 8:
+//     4 x 512^2 0.218 : 0.206, 3 x 400^2 0.122 : 0.163.
+//   m > 8: twice as many threads per patch while the CTAs are few (U = 120: 64^2,
+//     m = 16 0.078 -> 0.058 ms, m = 32 0.082 -> 0.063; above the lines the second
+//     reads of the bins' weights cost more, 4 x 256^2, m = 12 0.087 -> 0.135).  At
+//     m = 16 the two are close, and rounds of 4 and 5 CTAs per SM decide: 640 CTAs
+//     (10 x 256^2) 0.216 -> 0.181 ms.
+template <typename S, typename T, int M>
+dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool u_calc, cudaStream_t st, void *gt) {
+    if (!gt) gt = P->d_gt;
+    constexpr int NG = kFoldAdjNG<M>;
+    const long long nty = (P->ny + kAdjTY - 1) / kAdjTY, sms = P->num_sms;
+    const auto tiles = [&](int tx) { return (P->nx + tx - 1) / tx * nty; };
+    const auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    if constexpr (M <= 8) {
+        constexpr int ZS = M <= 4 ? 4 : 2, R = M <= 4 ? 23 : 17;
+        const long long one = tiles(32) * P->nz, many = tiles(32) * up(P->nz, ZS);
+        if (many >= 2 * sms && R * many < 10 * one && R * up(many, sms) < 10 * up(one, sms))
+            return fold_backproject_t<S, T, M, NG, ZS>(P, u, alpha, beta, u_calc, st, gt);
+    } else {
+        constexpr int few = M == 12 ? 4 : (M == 16 ? 10 : (M == 24 ? 6 : 8));  // quarters of CTAs per SM
+        const long long c = tiles(32 / NG) * P->nz, c2 = tiles(16 / NG) * P->nz;
+        if (4 * c <= few * sms || (M == 16 && 76 * up(c2, 5 * sms) < 100 * up(c, 4 * sms)))
+            return fold_backproject_t<S, T, M, 2 * NG, 1>(P, u, alpha, beta, u_calc, st, gt);
+    }
+    return fold_backproject_t<S, T, M, NG, 1>(P, u, alpha, beta, u_calc, st, gt);
 }
 
 // ===========================================================================

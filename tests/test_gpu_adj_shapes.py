@@ -43,3 +43,18 @@ def test_direct_two_slices_are_the_one_slice_bits(m, nx, ny, ns):
 
 def test_direct_two_slices_of_bf16_rows():
     _compare(47, 61, 75, 64, 33, 0.97, 7, dr.BF16, dr.DIRECT)
+
+
+# 304 CTAs of four (m <= 4) or two slices
+@pytest.mark.parametrize("m,nz", [(1, 151), (2, 152), (4, 151), (5, 75), (8, 76), (7, 75)])
+@pytest.mark.parametrize("prec", [dr.F32, dr.BF16])
+def test_folded_slices_per_thread_are_the_one_slice_bits(m, nz, prec):
+    _compare(45, 61, nz, 66, 60, 6, m, prec, dr.FOLD)
+
+
+# CTAs above the line from which a thread takes all (m <= 16) or half of a voxel's coefficients
+@pytest.mark.parametrize("m,nx,nz", [(10, 45, 40), (12, 64, 40), (16, 33, 100), (13, 50, 100), (24, 29, 60), (20, 32, 60),
+                                     (32, 17, 80), (27, 30, 80)])
+@pytest.mark.parametrize("prec", [dr.F32, dr.BF16])
+def test_folded_coefficients_per_thread_are_the_same_bits(m, nx, nz, prec):
+    _compare(nx, 31, nz, 66, 60, 6, m, prec, dr.FOLD)
