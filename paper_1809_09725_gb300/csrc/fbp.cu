@@ -114,7 +114,7 @@ static dr_status launch_filter_t(dr_plan *P, const void *g, cudaStream_t st) {
     const long long rows = (long long)P->nz * P->K, rg = (rows + R - 1) / R;
     const int nb4 = (P->ns + 3) / 4, tiles = (nb4 + 127) / 128, tb = (nb4 + tiles - 1) / tiles;
     // as many groups per CTA as its threads hold, while every SM gets two CTAs; in
-    // whole warps (idle lanes cost as much, most of all in FP64)
+    // whole warps (idle lanes cost as much)
     const int unit = std::max(1, 32 / tb);
     const long long fill = std::max<long long>(rg * tiles / (2 * P->num_sms) / unit, 1) * unit;
     const int groups = (int)std::min<long long>(std::min<long long>(kFbpThreads / tb, fill), rg);
@@ -132,14 +132,62 @@ static dr_status launch_filter_t(dr_plan *P, const void *g, cudaStream_t st) {
     return DR_OK;
 }
 
-// Eight rows per thread, unless that leaves SMs without a warp; then two, or in
-// FP64, whose pipe takes 59 clocks per warp and so wants a warp on each quarter
-// of an SM, one.
+// One row per CTA (grid-stride), one output per thread: shared memory holds the taps
+// h(n), n = -(ns - 1) .. ns - 1, and the row.
+constexpr int kFbpRowThreads = 256;
+template <typename S, typename T>
+__global__ void __launch_bounds__(kFbpRowThreads)
+    shepp_logan_row_kernel(const S *__restrict__ g, T *__restrict__ q, const T *__restrict__ taps, long long rows,
+                           int ns) {
+    extern __shared__ __align__(32) unsigned char fbp_smem[];
+    T *h = reinterpret_cast<T *>(fbp_smem);  // [2 ns - 1], h[i] = h(i - (ns - 1))
+    T *row = h + (2 * ns - 1);                // [ns]
+    for (int i = threadIdx.x; i < 2 * ns - 1; i += kFbpRowThreads) h[i] = taps[i];
+    for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
+        __syncthreads();  // previous row consumed
+        for (int i = threadIdx.x; i < ns; i += kFbpRowThreads) row[i] = ldc<T>(g + r * ns + i);
+        __syncthreads();
+        for (int b = threadIdx.x; b < ns; b += kFbpRowThreads) {
+            const T *hb = h + b + (ns - 1);  // hb[-b'] = h(b - b')
+            T acc = T(0);
+#pragma unroll 8
+            for (int bp = 0; bp < ns; ++bp) acc = fma(hb[-bp], row[bp], acc);
+            q[r * ns + b] = acc;
+        }
+    }
+}
+
+template <typename S, typename T>
+static dr_status launch_filter_row(dr_plan *P, const void *g, cudaStream_t st) {
+    const long long rows = (long long)P->nz * P->K;
+    const size_t smem = sizeof(T) * (size_t)(3 * P->ns - 1);
+    auto kern = shepp_logan_row_kernel<S, T>;
+    const dr_status s = allow_dynamic_smem((const void *)kern, smem);
+    if (s != DR_OK) return s;
+    int per_sm = 0;
+    DR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFbpRowThreads, smem));
+    const long long grid = std::min<long long>(rows, (long long)P->num_sms * std::max(per_sm, 1));
+    kern<<<(unsigned)grid, kFbpRowThreads, smem, st>>>((const S *)g, (T *)P->d_fbp_q, (const T *)P->d_fbp_taps, rows,
+                                                       P->ns);
+    DR_CUDA_TRY(cudaGetLastError());
+    return DR_OK;
+}
+
+// Eight rows per thread, unless that leaves SMs without a warp; then two.  One output
+// per thread in FP64, whose pipe (59 clocks per warp instruction) is the bound, so
+// that no register tile pays and its idle lanes and uneven CTAs cost (300 rows of
+// 257: 1.08 against 1.35 ms), and for a row per SM or fewer, where the longer chain
+// of four outputs would be all there is (30 rows of 128: 30 against 34 us).
 template <typename S, typename T>
 static dr_status launch_filter(dr_plan *P, const void *g, cudaStream_t st) {
-    const long long tasks = (long long)P->nz * P->K * ((P->ns + 3) / 4) / 8;
-    return tasks >= 32ll * P->num_sms ? launch_filter_t<S, T, 8>(P, g, st)
-                                      : launch_filter_t<S, T, sizeof(T) == 8 ? 1 : 2>(P, g, st);
+    const long long rows = (long long)P->nz * P->K;
+    if constexpr (sizeof(T) == 8) {
+        return launch_filter_row<S, T>(P, g, st);
+    } else {
+        if (rows <= P->num_sms && P->ns <= 512) return launch_filter_row<S, T>(P, g, st);
+        return rows * ((P->ns + 3) / 4) / 8 >= 32ll * P->num_sms ? launch_filter_t<S, T, 8>(P, g, st)
+                                                                  : launch_filter_t<S, T, 2>(P, g, st);
+    }
 }
 
 template <typename T>
