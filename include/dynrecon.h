@@ -215,9 +215,11 @@ dr_status dr_plan_set_fold_groups(dr_plan *plan, int group, int threads, int ray
 dr_status dr_plan_set_fold_march(dr_plan *plan, int nsplit, int async);
 
 /*
- * Fix the folded adjoint's distinct angles per pipeline stage (1..32; the
- * autotuner picks among 8, 7 and 6).  Each stage's folded-data windows share
- * a CTA's shared memory, so fewer angles per stage fit more CTAs on an SM.
+ * Fix the folded adjoint's distinct angles per pipeline stage (1..32, or as many
+ * as two stages of a CTA's 227 KB of shared memory hold, 28 and more; the
+ * autotuner picks among 8, 7 and 6 what fits 26 KB).  Each stage's folded-data
+ * windows share a CTA's shared memory, so fewer angles per stage fit more CTAs on
+ * an SM.
  * The angles are summed in the same order whatever the choice: results are
  * identical.  DR_EINVAL if the plan has no folded adjoint or angles is out of
  * range.
@@ -251,7 +253,7 @@ typedef struct {
     int fold2_lines;     /* two-kernel folded forward: strip lines */
     int fold2_split;     /* two-kernel folded forward: line chunks of the march */
     int fold2_async;     /* two-kernel folded forward: 1 if strips are double-buffered with cp.async */
-    int fold_adj_angles; /* folded adjoint: distinct angles per pipeline stage */
+    int fold_adj_angles; /* folded adjoint: distinct angles per pipeline stage (as set, or as tuned) */
     int fold2_angles;    /* two-kernel folded forward: distinct angles per CTA block */
     int fwd_variant_storage; /* variant dyn_radon_fwd uses now: 0, 1, 2, or 3 = the fold in two kernels with
                               * slices x coefficients on the lanes of a warp (automatic selection only) */

@@ -27,9 +27,9 @@
 namespace dr {
 
 constexpr int kFoldThreads = 256;
-constexpr int kFoldAdjP = 8;       // unique angles per adjoint pipeline stage (default; at most 32)
 constexpr int kFoldAdjStages = 2;
-constexpr int kFoldAdjWin = 26 * 1024;  // bytes of windows per stage, at most (four CTAs per SM)
+constexpr int kFoldAdjWin = 26 * 1024;  // bytes of windows per stage, at most, by default (four CTAs per SM)
+constexpr int kFoldAdjSmem = 227 * 1024;  // bytes of all stages where the caller chose the angles per stage
 
 // Padded coefficient stride in shared memory and in the folded data:
 // multiples of 4 floats (16-byte vectors, TMA rows) whose pattern of
@@ -1252,9 +1252,17 @@ dr_status fold_backproject_t(dr_plan *P, void *u, double alpha, double beta, boo
     // angles per pipeline stage: fewer shrink the windows' shared memory so that
     // more CTAs fit on an SM (the angles are summed in the same order)
     constexpr int row_bytes = Sh::WIN * (int)sizeof(T);
-    const int pp = std::max(1, std::min(std::min(32, P->fold_adj_pp), kFoldAdjWin / (ZS * row_bytes)));
-    const size_t stage = (size_t)pp * ZS * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128);
-    const size_t smem = stage * kFoldAdjStages + 128;
+    const auto bytes = [&](int pp) {
+        return kFoldAdjStages * ((size_t)pp * ZS * row_bytes + 128 * ((pp * sizeof(FoldPrm) + 127) / 128)) + 128;
+    };
+    int pp = std::max(1, std::min(32, P->fold_adj_pp));
+    if (P->fold_adj_pp_set) {
+        while (pp > 1 && bytes(pp) > kFoldAdjSmem) --pp;
+    } else {
+        pp = std::max(1, std::min(pp, kFoldAdjWin / (ZS * row_bytes)));
+    }
+    P->fold_adj_pp_used = pp;
+    const size_t smem = bytes(pp);
     auto kern = fold_adj_kernel<S, T, M, NG, ZS>;
     {
         dr_status s = allow_dynamic_smem((const void *)kern, smem);

@@ -632,14 +632,17 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
         // folded adjoint: distinct angles per pipeline stage (8, 7, 6: smaller
         // windows let more CTAs share an SM; the summation order is the same)
         int best_pp = 8;
+        P->fold_adj_pp_set = false;
+        P->fold_adj_pp_used = 32;
         for (int pp : {8, 7, 6}) {
+            if (pp >= P->fold_adj_pp_used) continue;  // (a stage held no more: the same launch)
             P->fold_adj_pp = pp;
             double t = 1e30;
             dr_status s = time_adj(1, t);
             if (s != DR_OK) return s;
             if (t < ms[3]) {
                 ms[3] = t;
-                best_pp = pp;
+                best_pp = P->fold_adj_pp_used;
             }
         }
         P->fold_adj_pp = best_pp;
@@ -853,6 +856,7 @@ dr_status dr_plan_set_fold_adj_stage(dr_plan *P, int angles) {
     if (P->fold_U == 0) return fail(DR_EINVAL, "dr_plan_set_fold_adj_stage: no folded adjoint");
     if (angles < 1 || angles > 32) return fail(DR_EINVAL, "dr_plan_set_fold_adj_stage: angles must be 1..32");
     P->fold_adj_pp = angles;
+    P->fold_adj_pp_set = true;
     return DR_OK;
 }
 

@@ -110,3 +110,14 @@ def test_timing_keeps_nothing_of_the_kernels_that_lost(size, prec):
         _pair(plan)
         held.append(plan.device_bytes())
     assert held[0] == held[1]
+
+
+@pytest.mark.parametrize("size,most", [((256, 256, 16, 256, 360, 4, 8), 6), ((256, 256, 16, 256, 360, 4, 16), 7)])
+def test_tuned_angles_per_stage_are_what_a_stage_holds(size, most):
+    """26 KB of windows: six angles of two slices with m = 8 (2 KB each), seven with
+    m = 16 (3.5 KB).  A caller's own choice is kept as it is given."""
+    plan = _plan(*size)
+    plan.autotune()
+    assert 6 <= plan.info()["fold_adj_angles"] <= most
+    plan.set_fold_adj_stage(12)
+    assert plan.info()["fold_adj_angles"] == 12
