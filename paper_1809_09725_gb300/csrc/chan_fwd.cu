@@ -27,8 +27,9 @@
 // EO: the same march in the order of the thread-per-ray kernels (a sample's even
 // pixel is added before its odd one): the even and the odd pixel keep their own
 // registers, and the lanes work out weights and steps of a line's rays side by
-// side.  Bit for bit the fold in two kernels, so the solvers can run on it; 0.44 ms
-// (three line chunks) and 8.5 ms on the two volumes above.
+// side.  Bit for bit the fold in two kernels, so the solvers can run on it, in that
+// fold's line chunks: 0.54 ms with its one on the first volume above (0.44 with three,
+// which would round differently) and 8.5 ms on the second.
 #include <algorithm>
 #include <cmath>
 #include <vector>

@@ -62,7 +62,7 @@ dr_status ensure_split_scratch(dr_plan *P, size_t bytes) {
 // Hold exactly what the choices need (trials of the autotuner grew it).
 static dr_status trim_split_scratch(dr_plan *P) {
     const size_t keep = split_bytes(P);
-    if (!P->d_ru_split || P->ru_split_bytes == keep) return DR_OK;
+    if (!P->d_ru_split || P->ru_split_bytes == keep || P->split_off) return DR_OK;
     cudaFree(P->d_ru_split);
     P->d_ru_split = nullptr;
     P->ru_split_bytes = 0;
@@ -649,7 +649,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
     }
     // the channel kernel against the fastest of the others (its trials may need
     // more partial sums than were chosen above)
-    if (P->chan.V && P->d_ru_split) {
+    if (P->chan.V && P->d_ru_split && !P->split_off) {
         cudaFree(P->d_ru_split);
         P->d_ru_split = nullptr;
         P->ru_split_bytes = 0;
@@ -731,8 +731,8 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
 // they run on the kernels of the thread-per-ray forms).
 static void hold_channel_scratch(dr_plan *P) {
     const ChanPlan &c = P->chan;
-    if (c.fwd || c.fwd_st) chan_fwd_ready(P, c.nsplit, P->graph_stream);
-    if (c.eo) chan_fwd_ready(P, fold2_chunks(P), P->graph_stream);
+    if (c.fwd || c.fwd_st) chan_fwd_ready(P, c.nsplit, P->stream);  // (not while that is being recorded)
+    if (c.eo) chan_fwd_ready(P, fold2_chunks(P), P->stream);
 }
 
 }  // namespace dr

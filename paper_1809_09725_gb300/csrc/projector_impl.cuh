@@ -303,9 +303,8 @@ enum AdjStaging { kAdjPlain, kAdjTma, kAdjCpAsync };
 //   4 x 256^2, K = 901, m = 32, rows of 257: 0.781 -> 0.617 ms
 //   16 x 256^2, K = 901, m = 16:             1.344 -> 1.108 ms
 //   6 x 128^2, K = 721, m = 8 (one slice):   0.154 -> 0.123 ms
-//   9 x 203 x 187, K = 721, m = 7, rows of 251: 0.314 -> 0.287 ms; two of three
-//   issue slots are used, by ten warps per SM (one slice per thread: 0.289 ms,
-//   twice the warps and 20 % more instructions)
+//   9 x 203 x 187, K = 721, m = 7, rows of 251: 0.314 -> 0.294 ms (one slice by the
+//   rule below; two take 0.287)
 // CTAs per SM asked for.  One slice: as many as the registers of the sums allow (64
 // to 72 of them); with five, a grid of 1024 CTAs (4 x 256^2, m = 12) no longer fits
 // the chip at once, 0.281 against 0.247 ms.  FP64: four or five, as the one-slice

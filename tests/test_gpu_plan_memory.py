@@ -121,3 +121,20 @@ def test_tuned_angles_per_stage_are_what_a_stage_holds(size, most):
     assert 6 <= plan.info()["fold_adj_angles"] <= most
     plan.set_fold_adj_stage(12)
     assert plan.info()["fold_adj_angles"] == 12
+
+
+def test_slab_solve_leaves_partial_sums_where_they_are():
+    """A slab-streamed solve that tunes its plan neither frees nor replaces the buffer
+    of partial sums that an earlier forward, perhaps recorded into a graph, wrote to."""
+    nz, K, n = 8, 192, 64
+    plan = _plan(n, n, nz, n, K, 8, 4)
+    plan.set_fold_march(3)
+    plan.set_variant(dr.FOLD2, dr.FOLD)
+    _pair(plan)
+    held = plan.device_bytes()
+    plan.set_variant(-1, -1)
+    g = synth.random_g(synth.rng_for(4972), nz, K, n).astype(np.float32)
+    u = np.zeros(plan.u_shape(), dtype=np.float32)
+    dr.cp_solve_slabs(plan, g, u, dr.solve_params(dr.CHAMBOLLE_POCK, iters=1, lambda1=0.05, lambda2=1.0, op_norm=60.0), 3)
+    assert plan.info()["tuned"] == 1
+    assert plan.device_bytes() == held
