@@ -15,11 +15,12 @@
 // ray's upper one, or (the carry of the position's fraction) one pixel
 // further, which is then read too.
 //
-// Bound by issue and shared memory together (ncu, 16 x 256^2, m = 8, 180
-// distinct angles: 71 % of the issue slots, 70 % of the shared-memory pipe; the
-// thread-per-ray kernels reach 90 % of that pipe with 1.7 times the bytes).
+// Bound by issue and shared memory together (ncu: 64 % of the issue slots and 61 % of
+// the shared-memory pipe on 16 x 256^2, m = 8, 180 distinct angles; 80 and 67 % on
+// 4 x 1024^2, m = 16; the thread-per-ray kernels reach 90 % of that pipe with 1.7
+// times the bytes).
 // Forward of 16 x 256^2, K = 1800, m = 8: 0.500 -> 0.373 ms; 8 x 1024^2,
-// K = 6000, m = 16: 16.3 -> 7.1 ms (0.13 -> 0.28 of the FP32 multiply-add
+// K = 6000, m = 16: 16.3 -> 7.25 ms (0.13 -> 0.28 of the FP32 multiply-add
 // rate).  Tried and slower: packed multiply-adds (0.405 ms: the copies that
 // pair the weights), a real branch instead of the predicated read (0.387 ms),
 // two lines at a time (0.390 ms with 16 warps, against 0.396 ms).

@@ -703,9 +703,10 @@ __global__ void __launch_bounds__(kRedThreads)
 //
 // Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.296 ms;
 // 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.49 ms.  Shared memory, 90 % busy with
-// pairs, is at 65 %; what bounds it now is issue (56 % of the slots) together
-// with the skew of a CTA's warps at the stage barrier (24 % of the stalls; three
-// stages on mbarriers without it measured 0.300 and 6.62 ms).
+// pairs, is at 61 % (m = 8) and 69 % (m = 16); what bounds it now is issue (59 and
+// 62 % of the slots) together with the skew of a CTA's warps at the stage barrier (a
+// quarter of the stalls; three stages on mbarriers without it measured 0.300 and
+// 6.62 ms).
 struct alignas(16) FoldPrm {
     float c, s, c16, e0;  // cos, sin, 16 cos, 1/cm - 1/(2 cm^2)  (cm = max(|c|, |s|))
     float inv_c2;           // 1/cm^2

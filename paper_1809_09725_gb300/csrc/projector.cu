@@ -238,6 +238,7 @@ dr_status autotune(dr_plan *P, void *u_scratch, void *g_scratch) {
             P->fold2_async = it->second.f2_async;
             P->fold2_async_st = it->second.f2_async_st;
             P->fold_adj_pp = it->second.adj_pp;
+            P->fold_adj_pp_set = false;
             P->fold2_bv = it->second.f2_bv;
             P->chan.fwd = it->second.chan_fwd;
             P->chan.fwd_st = it->second.chan_fwd_st;
