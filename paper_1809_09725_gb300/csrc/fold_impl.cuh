@@ -743,10 +743,11 @@ struct FoldAdjShape {
 
 // Resident CTAs asked for: 4 ZS MC sums, 11 weight pairs and 4 bins per thread.
 // (With five for m = 5 to 8 smaller grids are 4 to 6 % faster, but 761 to 912 CTAs
-// take a second round: 7 x 256^2, m = 8, U = 120 0.126 ms, with six 0.119.)
+// take a second round: 7 x 256^2, m = 8, U = 120 0.126 ms, with six 0.119; the same
+// holds of two threads a patch at m = 16: 2 x 327^2, U = 258 0.256 and 0.229 ms.)
 __host__ __device__ constexpr int fold_adj_min_blocks(int M, int NG, int ZS) {
     const int sums = ZS * M / NG;
-    return sums <= 4 ? 7 : (sums <= 8 ? (M <= 8 ? 6 : 5) : 4);
+    return sums <= 4 ? 7 : (sums <= 8 ? (M <= 8 || M == 16 ? 6 : 5) : 4);
 }
 
 // One thread of each CTA, when the CTA has read status[1] for the last time.
@@ -1288,8 +1289,10 @@ dr_status fold_backproject_t(dr_plan *P, void *u, double alpha, double beta, boo
 //   m > 8: twice as many threads per patch while the CTAs are few (U = 120: 64^2,
 //     m = 16 0.078 -> 0.058 ms, m = 32 0.082 -> 0.063; above the lines the second
 //     reads of the bins' weights cost more, 4 x 256^2, m = 12 0.087 -> 0.135).  At
-//     m = 16 the two are close, and rounds of 4 and 5 CTAs per SM decide: 640 CTAs
-//     (10 x 256^2) 0.216 -> 0.181 ms.
+//     m = 16 the two are within 7 % of one another, and what the last round of CTAs
+//     per SM costs decides: times for n CTAs on an SM, in us of U = 120, are those
+//     below (462 CTAs, 2 x 327^2, U = 258: 0.259 -> 0.229 ms; 640, 10 x 256^2, U = 120:
+//     0.216 -> 0.181).
 template <typename S, typename T, int M>
 dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool u_calc, cudaStream_t st, void *gt) {
     if (!gt) gt = P->d_gt;
@@ -1303,9 +1306,19 @@ dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool 
         if (many >= 2 * sms && R * many < 10 * one && R * up(many, sms) < 10 * up(one, sms))
             return fold_backproject_t<S, T, M, NG, ZS>(P, u, alpha, beta, u_calc, st, gt);
     } else {
-        constexpr int few = M == 12 ? 4 : (M == 16 ? 10 : (M == 24 ? 6 : 8));  // quarters of CTAs per SM
         const long long c = tiles(32 / NG) * P->nz, c2 = tiles(16 / NG) * P->nz;
-        if (4 * c <= few * sms || (M == 16 && 76 * up(c2, 5 * sms) < 100 * up(c, 4 * sms)))
+        bool fine;
+        if constexpr (M == 16) {
+            // all coefficients: full rounds of 103 and a last one of 1 to 4 CTAs; half: one
+            // round of up to 6 CTAs, then 13.6 each
+            constexpr int last[4] = {78, 86, 104, 135}, once[6] = {60, 67, 73, 82, 101, 118};
+            const long long n = up(c, sms), n2 = up(c2, sms);
+            fine = (n2 <= 6 ? 10 * once[n2 - 1] : 420 + 136 * n2) <= 1030 * ((n - 1) / 4) + 10 * last[(n - 1) % 4];
+        } else {
+            constexpr int few = M == 12 ? 4 : (M == 24 ? 6 : 8);  // quarters of CTAs per SM
+            fine = 4 * c <= few * sms;
+        }
+        if (fine)
             return fold_backproject_t<S, T, M, 2 * NG, 1>(P, u, alpha, beta, u_calc, st, gt);
     }
     return fold_backproject_t<S, T, M, NG, 1>(P, u, alpha, beta, u_calc, st, gt);
