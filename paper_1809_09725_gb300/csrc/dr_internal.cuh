@@ -277,7 +277,8 @@ struct dr_plan {
     double *d_partials = nullptr;
     unsigned *d_counters = nullptr;
     dr::DevScalars *d_scal = nullptr;
-    int *d_status = nullptr;          // [0] a wait gave up; [1] folded data not finite; [2] CTAs that are done with [1]
+    int *d_status = nullptr;          // [0] a wait gave up; [1], [2] folded data not finite, two launches in turn
+    int wild_slot = 0;                // which of the two the last launch took
     size_t table_bytes = 0;
     // FBP initial guess scratch (allocated on first use, fbp.cu)
     void *d_fbp_taps = nullptr;  // [2 ns - 1] T, Shepp-Logan taps

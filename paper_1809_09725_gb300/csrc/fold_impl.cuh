@@ -597,22 +597,29 @@ __global__ void __launch_bounds__(kRedThreads)
 // Adjoint, step 1: fold the data per unique angle
 //   gt[z][a][b][j] = sum_{k in group(a)} phi_j(t_k) g[z][k][flip_k(b)]
 // ===========================================================================
-// wild[0] = 1 if a folded row holds an infinity or a NaN: the back-projection
-// then takes each voxel's bins by themselves (0 x infinity would spread).
+// wild[slot] = 1 if a folded row holds an infinity or a NaN: the back-projection
+// that follows then takes each voxel's bins by themselves (0 x infinity would
+// spread).  The launches of a plan take two slots in turn, and each clears the one
+// of the next.  (A recorded launch keeps its slot: a note left in it by an earlier
+// replay costs time, not bits.)
 template <typename T, int N>
-__device__ __forceinline__ void note_wild(const T (&v)[N], int *wild) {
+__device__ __forceinline__ void note_wild(const T (&v)[N], int *wild, int slot) {
     T f = T(0);
 #pragma unroll
     for (int j = 0; j < N; ++j) f = fma(v[j], T(0), f);
-    if (f != T(0)) *(volatile int *)wild = 1;
+    if (f != T(0)) *(volatile int *)(wild + slot) = 1;
+}
+__device__ __forceinline__ void clear_next_wild(int *wild, int slot) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) wild[1 - slot] = 0;
 }
 
 template <typename S, typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
     fold_data_kernel(const S *__restrict__ g, T *__restrict__ gt, const int *__restrict__ start,
                      const int *__restrict__ member, const T *__restrict__ phip, int nz, int U, int ns, int K, int MP,
-                     int *wild) {
+                     int *wild, int slot) {
     constexpr int MS = fold_ms(M);
+    clear_next_wild(wild, slot);
     const size_t n = (size_t)nz * U * ns;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const int b = (int)(i % ns);
@@ -656,7 +663,7 @@ __global__ void __launch_bounds__(kRedThreads)
                 }
             }
         }
-        note_wild(acc, wild);
+        note_wild(acc, wild, slot);
         T *dst = gt + i * MS;
         if constexpr ((MS % 4) == 0 && sizeof(T) == 4) {
             float v[MS];
@@ -691,8 +698,7 @@ __global__ void __launch_bounds__(kRedThreads)
 // or cosine exceeds 0.99999, where the rounding of two positions could put
 // neighbouring taps two bins apart, read each voxel's two bins by themselves (a
 // CTA-uniform test per angle), and so do all angles when the kernel that wrote
-// the folded data found an infinity or a NaN in it (status[1]; the last CTA to
-// finish, counted in status[2], clears it for the next call).
+// the folded data found an infinity or a NaN in it (*wild).
 // A quarter warp's lanes are 4 x 2 patches: their lowest bins span at most
 // 6 |cos| + 2 |sin| < 8 bins, and rows of an odd number of 16-byte slots then
 // never collide (lanes on the same bin share one broadcast).
@@ -701,8 +707,8 @@ __global__ void __launch_bounds__(kRedThreads)
 // (|position| <= 18 bins: the weights are exact to about 1e-6); a tile is one
 // or two of them.
 //
-// Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.296 ms;
-// 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.49 ms.  Shared memory, 90 % busy with
+// Measured (data fold included): 16 x 256^2, K = 1800, m = 8: 0.351 -> 0.293 ms;
+// 8 x 1024^2, K = 6000, m = 16: 7.83 -> 6.64 ms.  Shared memory, 90 % busy with
 // pairs, is at 61 % (m = 8) and 69 % (m = 16); what bounds it now is issue (59 and
 // 62 % of the slots) together with the skew of a CTA's warps at the stage barrier (a
 // quarter of the stalls; three stages on mbarriers without it measured 0.300 and
@@ -750,18 +756,11 @@ __host__ __device__ constexpr int fold_adj_min_blocks(int M, int NG, int ZS) {
     return sums <= 4 ? 7 : (sums <= 8 ? (M <= 8 || M == 16 ? 6 : 5) : 4);
 }
 
-// One thread of each CTA, when the CTA has read status[1] for the last time.
-__device__ __forceinline__ void fold_adj_done(int *status) {
-    __threadfence();
-    const unsigned last = gridDim.x * gridDim.y - 1;
-    if (atomicInc(reinterpret_cast<unsigned *>(status + 2), last) == last) *(volatile int *)(status + 1) = 0;
-}
-
 template <typename S, typename T, int M, int NG_, int ZS>
 __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M, NG_, ZS))
     fold_adj_kernel(const __grid_constant__ CUtensorMap tm_gt, const FoldAng *__restrict__ ang,
                     S *__restrict__ u_s, T *__restrict__ u_c, int nx, int ny, int nz, int U, int U1, int m, T alpha,
-                    T beta, int *status, int PP, int vec) {
+                    T beta, int *status, const int *wild, int PP, int vec) {
     using Sh = FoldAdjShape<M, NG_>;
     constexpr int TX = Sh::TX, TY = kAdjTY, SX = Sh::SX, NG = Sh::NG, MC = Sh::MC;
     constexpr int NST = kFoldAdjStages;
@@ -838,8 +837,7 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M, NG_, ZS))
         if (lane != 0) mbar_arrive(&full[st]);
     };
 
-    // |sin| or |cos| above which the voxels of a patch go by themselves
-    const float axis = __ldcg(status + 1) != 0 ? -1.0f : 0.99999f;
+    const bool solo = __ldg(wild) != 0;
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) mbar_init(&full[s], 32);
         fence_mbar_init();
@@ -917,7 +915,7 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M, NG_, ZS))
                 w1 = fmaxf(0.0f, fmaf(d, ic2, h.w));
                 return __float_as_int(t) + idx;
             };
-            if (fabsf(ac) > axis || fabsf(as) > axis) {
+            if (solo || fabsf(ac) > 0.99999f || fabsf(as) > 0.99999f) {
                 // close to an axis, or bins that are not finite: each voxel's two bins by themselves
                 const float qv[4] = {qA, qB, qC, qD};
 #pragma unroll
@@ -987,13 +985,11 @@ __global__ void __launch_bounds__(kAdjThreads, fold_adj_min_blocks(M, NG_, ZS))
             if (tid == 0)
                 for (int s = kb; s < nkb && s < kb + NST; ++s)
                     mbar_wait_bounded(&full[s % NST], (unsigned)((s / NST) & 1), status, 100000000ull);
-            if (tid == 0) fold_adj_done(status);
             return;
         }
         // (the warps refill in turn: the others are already at the next stage)
         if (warp == (kb & 3) && kb + NST < nkb) issue(st, kb + NST);
     }
-    if (tid == 0) fold_adj_done(status);  // (behind the last stage's barrier)
     if (nk1 < nkb) flip();
 
 #pragma unroll
@@ -1235,7 +1231,7 @@ dr_status fold_adj_launch_t(dr_plan *P, const void *g, void *u, double alpha, do
     // step 1: fold the data into the scratch buffer
     fold_data_kernel<S, T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const S *)g, (T *)gt, P->d_fold_start, P->d_fold_member, (const T *)P->d_PhiP, P->nz, P->fold_U, P->ns,
-        P->K, P->MP, P->d_status + 1);
+        P->K, P->MP, P->d_status + 1, P->wild_slot ^= 1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_data_kernel launch");
     return fold_backproject<S, T, M>(P, u, alpha, beta, u_calc, st, gt);
@@ -1273,7 +1269,8 @@ dr_status fold_backproject_t(dr_plan *P, void *u, double alpha, double beta, boo
     const int ntx = (P->nx + Sh::TX - 1) / Sh::TX, nty = (P->ny + kAdjTY - 1) / kAdjTY;
     dim3 grid(ntx * nty, (P->nz + ZS - 1) / ZS);
     kern<<<grid, kAdjThreads, smem, st>>>(tm, P->d_fold_ang, u_calc ? nullptr : (S *)u, u_calc ? (T *)u : nullptr,
-                                          P->nx, P->ny, P->nz, P->fold_U, P->fold_U1, P->m, (T)alpha, (T)beta, P->d_status, pp,
+                                          P->nx, P->ny, P->nz, P->fold_U, P->fold_U1, P->m, (T)alpha, (T)beta, P->d_status,
+                                          P->d_status + 1 + P->wild_slot, pp,
                                           P->m == M && ((uintptr_t)u & 15u) == 0);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? DR_OK : cuda_fail(e, "fold_adj_kernel launch");
@@ -1336,7 +1333,8 @@ dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool 
 template <typename T, int M>
 __global__ void __launch_bounds__(kRedThreads)
     fold_gram_kernel(const T *ru, T *gt, const T *__restrict__ gram, int nz, int U, int ns, RowMap rin, int m,
-                     int nsplit, size_t split_stride, int *wild) {
+                     int nsplit, size_t split_stride, int *wild, int slot) {
+    clear_next_wild(wild, slot);
     // ru and gt may be the same buffer (one chunk): each thread reads its row
     // whole before writing it, so they are not declared __restrict__
     constexpr int MS = fold_ms(M);
@@ -1403,7 +1401,7 @@ __global__ void __launch_bounds__(kRedThreads)
             }
             ov[q] = acc;
         }
-        note_wild(ov, wild);
+        note_wild(ov, wild, slot);
         T *dst = gt + i * MS;
         if constexpr (V4 && MS % 4 == 0) {
 #pragma unroll
@@ -1431,7 +1429,7 @@ dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t 
     }
     fold_gram_kernel<T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows, P->m,
-        rs.nsplit, rs.split_stride, P->d_status + 1);
+        rs.nsplit, rs.split_stride, P->d_status + 1, P->wild_slot ^= 1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fold_gram_kernel launch");
     return fold_backproject<S, T, M>(P, y, 1.0, 0.0, true, st);
