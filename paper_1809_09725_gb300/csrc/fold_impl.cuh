@@ -512,7 +512,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == kFoldThreads ? fold_fwd_mi
 // bins of every projection k of angle a (at b, or ns-1-b for odd half-turns):
 // consecutive threads write consecutive bins of the same projection.
 // ===========================================================================
-template <typename S, typename T, int M>
+// (BLK: rows of several slices side by side, whose addresses take divisions; without
+// them a row is the i-th.  The divisions cost 1 us of the 37 of 6 x 128^2, m = 8, bf16.)
+template <typename S, typename T, int M, bool BLK>
 __global__ void __launch_bounds__(kRedThreads)
     fold_dist_kernel(const T *__restrict__ ru, S *__restrict__ out, const S *__restrict__ gm,
                      const int *__restrict__ start, const int *__restrict__ member, const T *__restrict__ phip,
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(kRedThreads)
         const int b = (int)(i % ns);
         const size_t za = i / ns;
         const int a = (int)(za % U), z = (int)(za / U);
-        const T *r = ru + row_at(rows, z, (size_t)a * ns + b);
+        const T *r = ru + (BLK ? row_at(rows, z, (size_t)a * ns + b) : i * rows.C);
         T rv[M];
         if constexpr (V4 && M % 4 == 0) {
 #pragma unroll
@@ -1210,7 +1212,8 @@ dr_status fold_fwd2_launch_t(dr_plan *P, const void *u, void *out, const void *g
                            : fold_static_dispatch<S, T, M>(P, u, st, rs);
         if (s != DR_OK) return s;
     }
-    fold_dist_kernel<S, T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
+    auto dist = rs.rows.spb > 1 ? fold_dist_kernel<S, T, M, true> : fold_dist_kernel<S, T, M, false>;
+    dist<<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const T *)rs.ru, (S *)out, (const S *)gm, P->d_fold_start, P->d_fold_member, (const T *)P->d_PhiP, P->nz,
         P->K, P->ns, P->fold_U, rs.rows, P->m, P->MP, mode, (T)sigma, rs.nsplit, rs.split_stride);
     cudaError_t e = cudaGetLastError();
@@ -1330,7 +1333,7 @@ dr_status fold_backproject(dr_plan *P, void *u, double alpha, double beta, bool 
 // the static transforms are mixed by G_a per (slice, angle, bin) and
 // back-projected, without the K projections in between.
 // ===========================================================================
-template <typename T, int M>
+template <typename T, int M, bool BLK>
 __global__ void __launch_bounds__(kRedThreads)
     fold_gram_kernel(const T *ru, T *gt, const T *__restrict__ gram, int nz, int U, int ns, RowMap rin, int m,
                      int nsplit, size_t split_stride, int *wild, int slot) {
@@ -1341,10 +1344,12 @@ __global__ void __launch_bounds__(kRedThreads)
     constexpr bool V4 = sizeof(T) == 4;
     const size_t n = (size_t)nz * U * ns;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int z = (int)(i / ((size_t)U * ns));
-        const size_t ab = i - (size_t)z * U * ns;
-        const int a = (int)(ab / ns);
-        const T *r = ru + row_at(rin, z, ab);
+        const int a = (int)((i / ns) % U);
+        const T *r = ru + i * rin.C;
+        if constexpr (BLK) {
+            const int z = (int)(i / ((size_t)U * ns));
+            r = ru + row_at(rin, z, i - (size_t)z * U * ns);
+        }
         T rv[M];
         if constexpr (V4 && M % 4 == 0) {
             // rows are multiples of 4 floats from 16-byte aligned bases
@@ -1427,7 +1432,8 @@ dr_status fold_normal_launch_t(dr_plan *P, const void *x, void *y, cudaStream_t 
         dr_status s = ensure_fold_scratch(P);
         if (s != DR_OK) return s;
     }
-    fold_gram_kernel<T, M><<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
+    auto gram = rs.rows.spb > 1 ? fold_gram_kernel<T, M, true> : fold_gram_kernel<T, M, false>;
+    gram<<<red_grid((size_t)P->nz * P->fold_U * P->ns), kRedThreads, 0, st>>>(
         (const T *)rs.ru, (T *)P->d_gt, (const T *)P->d_fold_gram, P->nz, P->fold_U, P->ns, rs.rows, P->m,
         rs.nsplit, rs.split_stride, P->d_status + 1, P->wild_slot ^= 1);
     cudaError_t e = cudaGetLastError();
